@@ -102,10 +102,14 @@ typedef struct {
                          log space on the float32 pipe, one table-driven loop per reaction class,
                          wdot accumulated in float pairs under a per-state power-of-two scale;
                          1 native float64 */
-  int tr_layout;      /* transport kernels' per-thread species vectors: 1 all in shared-memory
-                         columns; 2 the mole fractions in local memory (half the shared memory per
-                         thread, twice the resident warps); 0 (default) or 3 every vector in local
-                         memory (no shared memory; residency set by registers, 64 by default) */
+  int tr_layout;      /* transport kernels: 0 (default) the mixing sums as matrix products on the
+                         tensor cores (float16 digits of a 50-bit fixed-point product, added up in
+                         float pairs), 128 states per tile, for mechanisms with ln fits of up to
+                         160 species and with diff_mode, tr_mode, maxrreg and block at their
+                         defaults, else as 3; one thread per state with its species vectors: 1 all in
+                         shared-memory columns; 2 the mole fractions in local memory (half the
+                         shared memory per thread, twice the resident warps); 3 every vector in
+                         local memory (no shared memory; residency set by registers, 64 by default) */
   int maxrreg;        /* register cap per thread for the generated kernels; 0 = compiler choice */
   int block;          /* threads per block; 0 = 128 */
   int lazy;           /* 0: compile the production-rate, thermo and transport kernels at load
@@ -199,7 +203,9 @@ kx_status kx_thermo(kx_handle h, const double* T, const double* p, const double*
  * Pa s, Mathur conductivity lambda[n] in W/(m K) and diffusion coefficients
  * Dk[N_s][ld] in m^2/s (Eq. (mix_diff)), from the ln T polynomial fits of
  * ln eta_k, ln lambda_k and ln D_kj (Sec. A.3.4), D_kj scaled by p_atm/p.
- * A species whose partners all have X_j = 0 gets its self-diffusion D_kk. */
+ * A species whose partners all have X_j = 0 gets its self-diffusion D_kk.
+ * The default kernels hold the fits' temperature dependence for 200 to 4000 K;
+ * states outside are evaluated pair by pair (slower, the same accuracy). */
 kx_status kx_transport(kx_handle h, const double* T, const double* p, const double* Y, int64_t ld,
                        double* mu, double* lambda, double* Dk, int64_t n, kx_precision precision, void* stream);
 

@@ -54,7 +54,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         if src.endswith(".cu"):
             cmd = ["nvcc", "-c", "-O2", "-std=c++17", "-Xcompiler", "-fPIC", "-lineinfo", *ARCH, *inc, src, "-o", obj]
         else:
-            cmd = ["g++", "-c", "-O2", "-std=c++17", "-fPIC", "-Wall", *inc, src, "-o", obj]
+            cmd = ["g++", "-c", "-O2", "-std=c++17", "-fPIC", "-Wall", "-ffp-contract=off", *inc, src, "-o", obj]
         jobs.append((cmd, obj))
 
     def run(cmd):

@@ -59,6 +59,8 @@ struct Kernel {
   int max_blocks = 0;          // resident blocks for a persistent grid (per device 0 at load)
   int blocks_per_sm = 0;       // resident blocks per SM
   int smem = 0;                // dynamic shared memory per block, bytes
+  int threads = 0;             // threads per block
+  int row_chunks = 1;          // blocks that may share one tile of states (gridDim.y)
   int states_per_block = 0;    // states one block serves per pass of its grid-stride loop (0: one per thread)
   double lane_use = 1.0;       // warp-cooperative kernels: lane use of their class rounds
   int device = -1;
@@ -150,8 +152,17 @@ void parse_ptxas_info(const std::string& log, int& regs, int& local) {
 // Emit + compile (or fetch from the cache) one kernel.  Host only.
 kx_status compile_kernel(kx_mech* h, Kernel& k) {
   auto t0 = std::chrono::steady_clock::now();
-  k.source = kx::emit_kernel(h->m, k.kind, k.eopt, k.entry, &k.ops);
+  kx::KernelShape shape;
+  k.ops = kx::OpCounts();
+  k.source = kx::emit_kernel(h->m, k.kind, k.eopt, k.entry, &k.ops, &shape);
   if (k.source.empty()) return fail(KX_ERR_UNSUPPORTED, "kernel " + k.name + " is not available");
+  k.threads = k.eopt.block;
+  if (shape.threads > 0) {
+    k.threads = shape.threads;
+    k.smem = shape.smem;
+    k.states_per_block = shape.states_per_block;
+    k.row_chunks = shape.row_chunks;
+  }
   std::vector<std::string> opts = {"--gpu-architecture=sm_103a", "-std=c++17", "-lineinfo", "--ptxas-options=-v"};
   if (h->opt.libmath) opts.push_back("-DKX_LIBMATH");
 
@@ -220,7 +231,7 @@ kx_status load_kernel(Kernel& k) {
     e = cudaKernelSetAttributeForDevice(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, k.smem, dev);
     if (e != cudaSuccess) return cuda_fail(e, "cudaKernelSetAttributeForDevice");
   }
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)k.fn, k.eopt.block, k.smem);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)k.fn, k.threads, k.smem);
   if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
   k.max_blocks = sms * (per_sm > 0 ? per_sm : 1);
   k.blocks_per_sm = per_sm > 0 ? per_sm : 1;
@@ -267,8 +278,10 @@ kx_status launch(kx_mech* h, const char* name, void** args, int64_t n, void* str
   // thermo and transport 0-10 % faster.
   const int64_t cap = k->states_per_block > 0 ? (int64_t)k->max_blocks : (int64_t)INT_MAX;
   const int grid = (int)std::min<int64_t>(want, cap);
+  // few tiles: the blocks of a column share a tile's rows
+  const int gy = std::max(1, std::min(k->row_chunks, k->max_blocks / grid));
   cudaError_t e =
-      cudaLaunchKernel((const void*)k->fn, dim3(grid), dim3(k->eopt.block), args, k->smem, (cudaStream_t)stream);
+      cudaLaunchKernel((const void*)k->fn, dim3(grid, gy), dim3(k->threads), args, k->smem, (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(e, "cudaLaunchKernel");
   return KX_OK;
 }
@@ -422,6 +435,9 @@ kx_status kx_load_mechanism(const char* path, const kx_options* opt, kx_handle* 
       if (b < 32) return fail(KX_ERR_UNSUPPORTED, "mechanism too large for the transport kernel");
       k->eopt.block = b;
       k->smem = per * b;
+      // every transport option at its default: the sums on the tensor cores where the mechanism allows it
+      const kx_options& q = h->opt;
+      k->eopt.tr_tensor = q.tr_layout == 0 && q.tr_mode == 0 && q.diff_mode == 0 && q.maxrreg == 0 && (!opt || opt->block == 0);
     }
     h->kernels.push_back(std::move(k));
   }

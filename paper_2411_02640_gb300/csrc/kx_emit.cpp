@@ -37,7 +37,10 @@
 //    exp(-G/RT) products with one division (kc_mode = 1); float64 exp/log
 //    of our own (table-driven, Tang's method).  Table-driven above 64
 //    species or 400 reactions.
-//  * Transport (emit_transport): loops over per-species and per-pair
+//  * Transport, default (kx_emit_tc.cpp): the mixing sums as matrix products
+//    on the tensor cores.
+//  * Transport, one thread per state (emit_transport; direct fits and the
+//    explicit transport options): loops over per-species and per-pair
 //    coefficient tables, double-float by default; Wilke's sum over
 //    unordered pairs (phi_jk from phi_kj), symmetric D_kj evaluated once per
 //    pair and added to both rows.
@@ -51,14 +54,13 @@
 // (emit_class_mixed_body; the fully unrolled form is emit_rates_mixed).
 #include <algorithm>
 #include <cmath>
-#include <cstdarg>
-#include <cstdio>
 #include <cstring>
 #include <map>
 #include <set>
 #include <sstream>
 #include <tuple>
 
+#include "kx_emit_text.h"
 #include "kx_internal.h"
 
 namespace kx {
@@ -612,55 +614,9 @@ __device__ __forceinline__ void kx_acc_add(kx_df& acc, int& s, kx_df m, int e) {
 
 namespace {
 
-// ------------------------------------------------------------------ text helpers
-std::string fmt(const char* f, ...) {
-  va_list ap, ap2;
-  va_start(ap, f);
-  va_copy(ap2, ap);
-  const int n = vsnprintf(nullptr, 0, f, ap);
-  va_end(ap);
-  std::string out(n > 0 ? n : 0, '\0');
-  if (n > 0) vsnprintf(&out[0], n + 1, f, ap2);
-  va_end(ap2);
-  return out;
-}
-
-// float64 literal that reads back bit-exactly
-std::string D(double v) {
-  if (std::isnan(v)) return "KX_NAN";
-  if (std::isinf(v)) return v > 0 ? "KX_INF" : "(-KX_INF)";
-  std::string s = fmt("%.17g", v);
-  if (s.find_first_of(".en") == std::string::npos) s += ".0";
-  return s[0] == '-' ? "(" + s + ")" : s;
-}
-
-// float32 literal (value rounded to float first)
-std::string F(double v) {
-  float f = (float)v;
-  if (std::isinf(f)) return v > 0 ? "__int_as_float(0x7f800000)" : "(-__int_as_float(0x7f800000))";
-  std::string s = fmt("%.9g", (double)f);
-  if (s.find_first_of(".en") == std::string::npos) s += ".0";
-  s += "f";
-  return s[0] == '-' ? "(" + s + ")" : s;
-}
-
-std::string fpair(double v) {
-  const float h = (float)v;
-  const float l = (float)(v - (double)h);
-  return F(h) + "," + F(l);
-}
-
-std::string DFc(double v) { return "kx_mk(" + fpair(v) + ")"; }
-
 // float32-pipe instruction estimates of the double-float primitives (for the
 // operation counts)
 constexpr double kDfAdd = 11, kDfMul = 7, kDfFma = 15, kDfMulf = 5, kDfDiv = 16, kDfExp = 30, kDfLog = 40;
-
-struct Out {
-  std::ostringstream o;
-  int ind = 1;
-  void operator()(const std::string& s) { o << std::string(2 * ind, ' ') << s << "\n"; }
-};
 
 bool is_small_int(double b) { return b == std::floor(b) && std::fabs(b) <= 4.0; }
 
@@ -2797,34 +2753,6 @@ void emit_thermo(Out& o, const Mechanism& m, OpCounts& c) {
 //        scaled by log2(e) so each property is one exp2.
 double wilke_a(const Mechanism& m, int k, int j) { return 1.0 / std::sqrt(8.0 * (1.0 + m.W[k] / m.W[j])); }
 
-// Double-double host arithmetic from error-free transformations (std::fma is exact IEEE arithmetic
-// on every host), so that the emitted constants are the same bits on every platform: long double is
-// 80-bit on x86-64 and 128-bit on aarch64.
-struct HostDD { double hi, lo; };
-HostDD hdd_norm(double a, double b) { const double s = a + b; return {s, b - (s - a)}; }
-HostDD hdd_add(HostDD a, HostDD b) {
-  const double s = a.hi + b.hi, bb = s - a.hi;
-  const double e = (a.hi - (s - bb)) + (b.hi - bb);
-  return hdd_norm(s, e + a.lo + b.lo);
-}
-HostDD hdd_mul(HostDD a, HostDD b) {
-  const double p = a.hi * b.hi;
-  return hdd_norm(p, std::fma(a.hi, b.hi, -p) + (a.hi * b.lo + a.lo * b.hi));
-}
-
-// p(L) = sum c_n L^n re-expanded about L0: d_m = sum_{n>=m} C(n,m) c_n L0^(n-m), in double-double
-void shift_poly(const double* cf, double L0, double scale, double out[5]) {
-  static const double binom[5][5] = {{1, 0, 0, 0, 0}, {1, 1, 0, 0, 0}, {1, 2, 1, 0, 0}, {1, 3, 3, 1, 0}, {1, 4, 6, 4, 1}};
-  HostDD pw[5] = {{1.0, 0.0}};
-  for (int k = 1; k < 5; ++k) pw[k] = hdd_mul(pw[k - 1], {L0, 0.0});
-  for (int mm = 0; mm < 5; ++mm) {
-    HostDD d = {0.0, 0.0};
-    for (int n = mm; n < 5; ++n) d = hdd_add(d, hdd_mul(hdd_mul({binom[n][mm], 0.0}, {cf[n], 0.0}), pw[n - mm]));
-    d = hdd_mul(d, {scale, 0.0});
-    out[mm] = d.hi + d.lo;
-  }
-}
-
 struct TrMode {
   enum { F64, DF, F32 } kind;
   const char* ty;     // arithmetic type
@@ -4374,8 +4302,12 @@ std::string emit_vjp_wc_kernel(const Mechanism& m, const EmitOptions& opt, const
 }
 
 std::string emit_kernel(const Mechanism& m, KernelKind kind, const EmitOptions& opt, const std::string& entry,
-                        OpCounts* counts) {
+                        OpCounts* counts, KernelShape* shape) {
   if (vjp_is_wc(m, kind, opt)) return emit_vjp_wc_kernel(m, opt, entry, counts);
+  if (kind == KernelKind::Transport && opt.tr_tensor) {
+    const std::string tc = emit_transport_tc(m, opt, entry, counts, shape);
+    if (!tc.empty()) return tc;
+  }
   OpCounts c;
   Out body, globals;
   body.ind = 2;

@@ -80,6 +80,7 @@ struct EmitOptions {
   int vjp_form = 0;         // double-float adjoint, d/dC_k: 0 rate mantissa times a per-state reciprocal
                             // concentration, 1 one log-space exponential per entry
   int vjp_layout = 0;       // double-float adjoint: 0/1 thread per state, 2 warp-cooperative
+  bool tr_tensor = false;   // transport sums on the tensor cores where the mechanism allows it
   int rates_negligible = 0; // double-float rates: 0 float32 for reactions negligible in every state of a warp, 1 never
 };
 
@@ -99,9 +100,20 @@ struct OpCounts {
   double fp64 = 0, fp32 = 0, exp64 = 0, log64 = 0, div64 = 0, exp32 = 0, log32 = 0, div32 = 0;
 };
 
+// Launch shape of a kernel that fixes its own (threads 0: the options' block, one state per thread).
+struct KernelShape {
+  int threads = 0, smem = 0, states_per_block = 0;
+  int row_chunks = 1;      // blocks that can share a tile's rows (gridDim.y)
+};
+
 // CUDA C++ source of one kernel, entry point named `entry`.
 std::string emit_kernel(const Mechanism& m, KernelKind kind, const EmitOptions& opt, const std::string& entry,
-                        OpCounts* counts);
+                        OpCounts* counts, KernelShape* shape = nullptr);
+
+// The tensor-core transport kernel (kx_emit_tc.cpp); empty where the mechanism does not allow it
+// (direct fits, too many species for tensor memory, too many basis functions).
+std::string emit_transport_tc(const Mechanism& m, const EmitOptions& opt, const std::string& entry, OpCounts* counts,
+                              KernelShape* shape);
 
 // Global scratch bytes per thread of the float-pair rate kernel built with
 // EmitOptions::scratch ({ln |C|, mu} float4 and a float-pair accumulator per species).
