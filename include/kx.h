@@ -189,7 +189,9 @@ kx_status kx_production_rates(kx_handle h, const double* T, const double* p, con
 
 /* Rates of progress q[N_r][ld] of every reaction, R_i = c_i r_i (Sec. A.2),
  * the per-reaction quantity the paper validates as "reaction rates"
- * (Table 3). */
+ * (Table 3).  Small batches (below about 52000 u^1.3 states, u as in
+ * kx_options.rates_layout; KX_MIXED 0.6 of that) run the warp-cooperative
+ * float-pair kernel for either precision. */
 kx_status kx_rates_of_progress(kx_handle h, const double* T, const double* p, const double* Y, int64_t ld,
                                double* q, int64_t n, kx_precision precision, void* stream);
 
@@ -288,9 +290,11 @@ kx_status kx_production_rates_noalloc(kx_handle h, const double* T, const double
  * are "wdot_fp64", "wdot_mixed", "rop_fp64", "rop_mixed", "thermo",
  * "visc_fp64", "visc_mixed", "diff_fp64", "diff_mixed", "vjp" and
  * "wdot_fp64_noalloc" (the kernel of kx_production_rates_noalloc),
- * "wdot_fp64_wc" (the warp-cooperative production-rate kernel) and
+ * "wdot_fp64_wc" (the warp-cooperative production-rate kernel),
  * "vjp_wc" (the warp-cooperative adjoint of small batches; absent when
- * kx_options.vjp_layout or rates_arith fixes the adjoint kernel).  Any
+ * kx_options.vjp_layout or rates_arith fixes the adjoint kernel) and
+ * "rop_fp64_wc" (the warp-cooperative rates of progress of small batches;
+ * absent when rates_layout, rates_arith or rates_mode is not 0).  Any
  * output pointer may be NULL.  registers and local_bytes: per thread, from
  * the compiler's report (local_bytes is the stack frame: local arrays and
  * register spills, the local memory the driver backs for every resident

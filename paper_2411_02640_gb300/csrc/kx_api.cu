@@ -16,6 +16,7 @@
 #include <atomic>
 #include <chrono>
 #include <climits>
+#include <cmath>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -376,7 +377,7 @@ kx_status kx_load_mechanism(const char* path, const kx_options* opt, kx_handle* 
       {"diff_fp64", kx::KernelKind::Transport, false, 2}, {"visc_mixed", kx::KernelKind::Transport, true, 1},
       {"diff_mixed", kx::KernelKind::Transport, true, 2}, {"vjp", kx::KernelKind::Vjp, false, 0},
       {"wdot_fp64_noalloc", kx::KernelKind::Wdot, false, 0}, {"wdot_fp64_wc", kx::KernelKind::Wdot, false, 0},
-      {"vjp_wc", kx::KernelKind::Vjp, false, 0},
+      {"vjp_wc", kx::KernelKind::Vjp, false, 0},             {"rop_fp64_wc", kx::KernelKind::Rop, false, 0},
   };
   for (const Spec& sp : specs) {
     std::unique_ptr<Kernel> k(new Kernel());
@@ -400,6 +401,11 @@ kx_status kx_load_mechanism(const char* path, const kx_options* opt, kx_handle* 
     k->eopt.vjp_form = h->opt.vjp_form;
     k->eopt.vjp_layout = h->opt.vjp_layout;
     k->eopt.rates_negligible = h->opt.rates_negligible;
+    if (std::strcmp(sp.name, "rop_fp64_wc") == 0) {
+      // the warp-cooperative rates of progress beside the default ones, for small batches
+      if (h->opt.rates_layout != 0 || h->opt.rates_arith == 1 || h->opt.rates_mode != 0) continue;
+      k->eopt.rop_wc = true;
+    }
     const bool vjp_wc_spec = std::strcmp(sp.name, "vjp_wc") == 0;
     if (vjp_wc_spec) {
       // the warp-cooperative adjoint beside the default one, for small batches
@@ -419,6 +425,7 @@ kx_status kx_load_mechanism(const char* path, const kx_options* opt, kx_handle* 
     }
     if (kx::wdot_is_wc(h->m, sp.kind, k->eopt)) {
       const kx::WcShape w = kx::wdot_wc_shape(h->m, k->eopt);
+      if (w.smem_per_block > 200 * 1024 && k->eopt.rop_wc) continue;   // too large: the default kernel serves every batch
       if (w.smem_per_block > 200 * 1024)
         return fail(KX_ERR_UNSUPPORTED, "warp-cooperative rate kernel: one block's shared memory exceeds 200 KB "
                                         "(choose a smaller rates_group or rates_layout 1)");
@@ -438,6 +445,7 @@ kx_status kx_load_mechanism(const char* path, const kx_options* opt, kx_handle* 
       // every transport option at its default: the sums on the tensor cores where the mechanism allows it
       const kx_options& q = h->opt;
       k->eopt.tr_tensor = q.tr_layout == 0 && q.tr_mode == 0 && q.diff_mode == 0 && q.maxrreg == 0 && (!opt || opt->block == 0);
+
     }
     h->kernels.push_back(std::move(k));
   }
@@ -502,6 +510,16 @@ kx_status kx_mechanism_info(kx_handle h, int* n_species, int* n_reactions, doubl
 
 namespace {
 
+// The batch size from which a thread-per-state kernel is the faster one, against the warp-cooperative kernel
+// `wc` of the same rates: the first takes one state's latency whatever the batch, the second its time per state
+// times the batch, which grows with the inverse of its lane use and of its resident warps.  Measured crossovers
+// of the rates of progress: 9/21 ~8k states (lane use 0.22, 24 warps per SM), 53/325 ~45k (0.92, 24), 160/900
+// ~31k (0.95, 16).
+int64_t small_batch_below(const Kernel& wc, double scale) {
+  const double warps = std::min(24, wc.blocks_per_sm * (wc.eopt.block / 32));
+  return (int64_t)(scale * 52000.0 * std::pow(wc.lane_use, 1.3) * warps / 24.0);
+}
+
 // The production-rate kernel for a batch of n states.  Small float64-accurate batches go to the
 // warp-cooperative kernel, whose warps share each state: the thread-per-state kernel would leave
 // SMs idle and take one state's whole latency.  The crossover, measured on GB300, sits near 48k
@@ -518,6 +536,20 @@ kx_status wdot_kernel_for(kx_mech* h, int64_t n, kx_precision precision, const c
   if (s != KX_OK) return s;
   const int64_t cap = (int64_t)tps->max_blocks * tps->eopt.block;
   if (n < std::min<int64_t>(cap, (int64_t)(49152.0 * wc->lane_use))) *name = "wdot_fp64_wc";
+  return KX_OK;
+}
+
+// The rates-of-progress kernel for a batch of n states: small batches go to the warp-cooperative kernel
+// (float pairs throughout, for either precision: a mixed call gets at least what it asked for).  53/325:
+// one thread per state 320-390 us (mixed 219-274) up to 32k states; warp-cooperative 20 us at 997 states,
+// 121 at 16383, 269 at 32768.
+kx_status rop_kernel_for(kx_mech* h, int64_t n, kx_precision precision, const char** name) {
+  *name = precision == KX_FP64 ? "rop_fp64" : "rop_mixed";
+  Kernel* wc = find_kernel(h, "rop_fp64_wc");
+  if (!wc) return KX_OK;
+  kx_status s = ensure_ready(h, *wc);
+  if (s != KX_OK) return s;
+  if (n < small_batch_below(*wc, precision == KX_FP64 ? 1.0 : 0.6)) *name = "rop_fp64_wc";
   return KX_OK;
 }
 
@@ -639,7 +671,9 @@ kx_status kx_rates_of_progress(kx_handle h, const double* T, const double* p, co
   if (n == 0) return KX_OK;
   long long ldl = ld, nl = n;
   void* args[] = {&T, &p, &Y, &ldl, &q, &nl};
-  return launch(h, precision == KX_FP64 ? "rop_fp64" : "rop_mixed", args, n, stream);
+  const char* name = nullptr;
+  if ((s = rop_kernel_for(h, n, precision, &name)) != KX_OK) return s;
+  return launch(h, name, args, n, stream);
 }
 
 kx_status kx_thermo(kx_handle h, const double* T, const double* p, const double* Y, int64_t ld, double* cp,

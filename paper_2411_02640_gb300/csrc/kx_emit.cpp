@@ -3247,7 +3247,7 @@ WcLayout wc_layout_of(const Mechanism& m, int group, int block) {
 }
 
 std::string emit_wdot_wc(const Mechanism& m, const EmitOptions& opt, const std::string& entry, OpCounts& c,
-                         Out& globals) {
+                         Out& globals, bool rop) {
   const int ns = m.ns, nr = m.nr();
   const WcLayout L = wc_layout_of(m, opt.rates_group, opt.block);
   const int G = L.G, NW32 = L.nw32, SVS = L.svs;
@@ -3470,7 +3470,7 @@ std::string emit_wdot_wc(const Mechanism& m, const EmitOptions& opt, const std::
       // the state's running largest power of two is a warp max of the lanes' own; a round whose
       // reactions all have both rates below 2^-40 of it takes float32 (the rate scaled by 2^-emx,
       // stored with the power of two emx)
-      const bool fastp = G == 1 && opt.rates_negligible == 0 && (d.kind == Kind::Elementary || d.kind == Kind::ThreeBody || fo);
+      const bool fastp = !rop && G == 1 && opt.rates_negligible == 0 && (d.kind == Kind::Elementary || d.kind == Kind::ThreeBody || fo);
       const int dnf = d.npr - d.nre;
       auto negbit0 = [&](int j) { return fmt("((nmg[k%d >> 5] >> (k%d & 31)) & 1)", j, j); };
       if (fastp) {
@@ -3641,6 +3641,25 @@ std::string emit_wdot_wc(const Mechanism& m, const EmitOptions& opt, const std::
   }
   --o.ind;
   o("}");
+  if (rop) {
+    // rates of progress: every reaction's mantissa and power of two written out as float64, consecutive
+    // lanes on the group's consecutive states
+    o("__syncwarp();");
+    o("#pragma unroll 4");
+    o(fmt("for (int p = lane; p < %d; p += 32) {", G * nr));
+    o(fmt("  const int g = p & %d, r = p >> %d;", G - 1, LG));
+    o("  const int flag = sci[g].y;");
+    o("  if (flag == 2) continue;");
+    o(fmt("  const float2 q = qm[%d * g + r];", nr));
+    o(fmt("  out_[(long long)r * ld + i0 + g] = flag == 1 ? KX_NAN : kx_df2d_s(kx_df_norm(kx_mk(q.x, q.y)), (int)qe[%d * g + r]);", nr));
+    o("}");
+    o(fmt("if (lane < %d && sci[lane].y == 1) atomicMin(&kx_bad_first, (unsigned long long)(i0 + lane));", G));
+    o("__syncwarp();");
+    --o.ind;
+    o("}");
+    c.fp64 += nr;
+    return o.o.str();
+  }
   // ---- 4. the largest exponent of each state (a warp max over its rates); rates scaled in place
   o("__syncwarp();");
   o(fmt("for (int g = 0; g < %d; ++g) {", G));
@@ -4214,6 +4233,7 @@ int transport_smem_per_thread(const Mechanism& m, bool mixed, int part, int layo
 // ------------------------------------------------------------------ kernels
 bool wdot_is_wc(const Mechanism& m, KernelKind kind, const EmitOptions& opt) {
   (void)m;
+  if (kind == KernelKind::Rop) return opt.rop_wc;
   return kind == KernelKind::Wdot && !opt.mixed && !opt.scratch && opt.rates_arith != 1 && opt.rates_layout == 2;
 }
 
@@ -4239,11 +4259,11 @@ WcShape wdot_wc_shape(const Mechanism& m, const EmitOptions& opt) {
 
 // The warp-cooperative production-rate kernel (emit_wdot_wc) with its own
 // grid-stride loop over groups of states.
-std::string emit_wc_kernel(const Mechanism& m, const EmitOptions& opt, const std::string& entry, OpCounts* counts) {
+std::string emit_wc_kernel(const Mechanism& m, const EmitOptions& opt, const std::string& entry, OpCounts* counts, bool rop) {
   OpCounts c;
   Out globals;
   globals.ind = 0;
-  const std::string body = emit_wdot_wc(m, opt, entry, c, globals);
+  const std::string body = emit_wdot_wc(m, opt, entry, c, globals, rop);
   if (body.empty()) return "";
   std::ostringstream s;
   s << "// mechanism " << m.name << ": " << m.ns << " species, " << m.nr() << " reactions\n";
@@ -4317,7 +4337,7 @@ std::string emit_kernel(const Mechanism& m, KernelKind kind, const EmitOptions& 
     case KernelKind::Wdot:
     case KernelKind::Rop: {
       const bool rop = kind == KernelKind::Rop;
-      if (wdot_is_wc(m, kind, opt)) return emit_wc_kernel(m, opt, entry, counts);
+      if (wdot_is_wc(m, kind, opt)) return emit_wc_kernel(m, opt, entry, counts, rop);
       outs = "double* __restrict__ out_";
       if (opt.scratch && !rop) outs += ", unsigned char* __restrict__ kx_scr, long long nthr";
       nan_fill = fmt("for (int k = 0; k < %d; ++k) out_[(long long)k * ld + i] = KX_NAN;", rop ? m.nr() : m.ns);
