@@ -445,7 +445,9 @@ kx_status kx_load_mechanism(const char* path, const kx_options* opt, kx_handle* 
       // every transport option at its default: the sums on the tensor cores where the mechanism allows it
       const kx_options& q = h->opt;
       k->eopt.tr_tensor = q.tr_layout == 0 && q.tr_mode == 0 && q.diff_mode == 0 && q.maxrreg == 0 && (!opt || opt->block == 0);
-
+    }
+    if (sp.kind == kx::KernelKind::Thermo) {
+      k->eopt.tr_tensor = h->opt.maxrreg == 0 && (!opt || opt->block == 0);
     }
     h->kernels.push_back(std::move(k));
   }

@@ -44,7 +44,10 @@
 //    coefficient tables, double-float by default; Wilke's sum over
 //    unordered pairs (phi_jk from phi_kj), symmetric D_kj evaluated once per
 //    pair and added to both rows.
-//  * Thermo (emit_thermo): two float-pair Horner evaluations per species.
+//  * Thermo, default (kx_emit_tc.cpp): the NASA-7 polynomials' mixture
+//    coefficients as a matrix product on the tensor cores; emit_thermo (more
+//    than four distinct T_mid, or explicit block or register options): two
+//    float-pair Horner evaluations per species.
 //
 // The mixed-precision production rates (KX_MIXED) run the same class loops
 // with a float32 body for the Arrhenius, third-body and falloff arithmetic;
@@ -4324,8 +4327,10 @@ std::string emit_vjp_wc_kernel(const Mechanism& m, const EmitOptions& opt, const
 std::string emit_kernel(const Mechanism& m, KernelKind kind, const EmitOptions& opt, const std::string& entry,
                         OpCounts* counts, KernelShape* shape) {
   if (vjp_is_wc(m, kind, opt)) return emit_vjp_wc_kernel(m, opt, entry, counts);
-  if (kind == KernelKind::Transport && opt.tr_tensor) {
-    const std::string tc = emit_transport_tc(m, opt, entry, counts, shape);
+  if ((kind == KernelKind::Transport || kind == KernelKind::Thermo) && opt.tr_tensor) {
+    EmitOptions q = opt;
+    if (kind == KernelKind::Thermo) q.part = 3;
+    const std::string tc = emit_transport_tc(m, q, entry, counts, shape);
     if (!tc.empty()) return tc;
   }
   OpCounts c;

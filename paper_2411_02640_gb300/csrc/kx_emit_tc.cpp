@@ -1,4 +1,4 @@
-// Emitter of the tensor-core transport kernels (tcgen05, sm_103a).
+// Emitter of the tensor-core transport and thermo kernels (tcgen05, sm_103a).
 //
 // The mixing sums of the transport properties are products of a state's mass
 // fractions with matrices that depend on temperature alone, and those are
@@ -30,6 +30,11 @@
 // 200-4000 K (or with non-finite Y) and rows whose sum is small beside the state's
 // largest v (a nearly pure state's own row) are evaluated pair by pair in float
 // pairs instead.
+//
+// Thermo (part 3) is the same with one stage: the mixture's polynomial coefficients,
+// per T_mid group and range, as rows of an exact basis (tc_thermo), then c_p and h per
+// state.  53/325: 39 -> 12 us up to 16k states (one thread per state took that state's
+// 53 x 11 dependent float-pair steps), 49152 states 39 -> 20 us; 160/900 121 -> 14 us.
 //
 // What bounds it (53/325, GB300): instruction issue and the latencies between the
 // stages of a tile (57-66 % of issue slots at four warps per scheduler; the matrix
@@ -228,6 +233,8 @@ struct Plan {
   std::vector<Stage> st;
   int acols = 0, dcols = 0, nbuf = 2, slots = 0, slot_bytes = 0, chunk_bytes = 0, chunks = 0;
   int smem = 0;
+  int red = 24;                            // rows of 128 values exchanged between the compute groups
+  std::vector<double> mids;                // thermo: the distinct T_mid
 };
 
 std::string hex64(unsigned long long v) { return fmt("0x%llxULL", v); }
@@ -235,7 +242,7 @@ std::string hex64(unsigned long long v) { return fmt("0x%llxULL", v); }
 bool make_plan(const Mechanism& m, const EmitOptions& opt, Plan& p) {
   p.mixed = opt.mixed;
   p.part = opt.part;
-  if (!tc_basis(m, opt.part, opt.mixed, p.b)) return false;
+  if (opt.part == 3 ? !tc_thermo(m, p.b, p.mids) : !tc_basis(m, opt.part, opt.mixed, p.b)) return false;
   const TcBasis& b = p.b;
   p.nd = opt.mixed ? 3 : 5;
   // digits that keep each set's dropped products near 2^-48 of the largest v (mixed: 2^-26)
@@ -288,7 +295,8 @@ bool make_plan(const Mechanism& m, const EmitOptions& opt, Plan& p) {
     p.st.push_back(s);
   }
   p.chunks = (b.rows + kRowsChunk - 1) / kRowsChunk;
-  const int fixed = (b.M + 1) * kStates * 8 + 24 * kStates * 8 + (b.M + 1) * 32 * 8 + p.chunks * kRowsChunk * 8 + b.K * 4 + 1024 +
+  if (opt.part == 3) p.red = 8 + kRowsChunk * p.chunks;
+  const int fixed = (b.M + 1) * kStates * 8 + p.red * kStates * 8 + (b.M + 1) * 32 * 8 + p.chunks * kRowsChunk * 8 + b.K * 4 + 1024 +
                     (b.K <= 64 ? b.K * kStates * 8 : 0);   // (the next tile's Y, for mechanisms small enough)
   p.slots = std::min(8, (200 * 1024 - fixed) / p.slot_bytes);
   p.slots = std::min(p.slots, std::max(2, (int)p.st.size() * p.chunks));
@@ -398,6 +406,23 @@ void emit_pairwise(std::ostringstream& s, const Mechanism& m, const Plan& p) {
       << "  const float2* t = kx_dc + 5 * (k * " << ns << " - k * (k - 1) / 2);\n"
       << "  const kx_df e = " << horner("t") << ";\n"
       << "  return kx_df2d(kx_df_exp(kx_mk(-e.hi, -e.lo))) * pr;\n}\n";
+    return;
+  }
+  if (p.part == 3) {
+    std::vector<double> a;
+    for (int k = 0; k < ns; ++k)
+      for (int rg = 0; rg < 2; ++rg)
+        for (int n = 0; n < 6; ++n) a.push_back(rg == 0 ? m.a_lo[7 * k + n] : m.a_hi[7 * k + n]);
+    s << "__device__ const double kx_nasa[" << a.size() << "] = {" << list(a, false) << "};\n";
+    s << "__device__ const double kx_tmid[" << ns << "] = {" << list(m.Tmid, false) << "};\n";
+    s << "__device__ __noinline__ double2 kx_thermo_state(const double* __restrict__ Y_, long long ld, long long i, double T) {\n"
+      << "  double cp = 0.0, h = 0.0;\n"
+      << "  for (int k = 0; k < " << ns << "; ++k) {\n"
+      << "    const double* a = kx_nasa + 12 * k + (T < kx_tmid[k] ? 0 : 6);\n"
+      << "    const double y = Y_[(long long)k * ld + i] * (" << D(R_U) << " / kx_w[k]);\n"
+      << "    cp = fma(y, fma(fma(fma(fma(a[4], T, a[3]), T, a[2]), T, a[1]), T, a[0]), cp);\n"
+      << "    h = fma(y, fma(fma(fma(fma(fma(a[4] * 0.2, T, a[3] * 0.25), T, a[2] / 3.0), T, a[1] * 0.5), T, a[0]), T, a[5]), h);\n"
+      << "  }\n  return make_double2(cp, h);\n}\n";
     return;
   }
   std::vector<double> pv, pl, wa, sq;
@@ -536,7 +561,7 @@ std::string emit_transport_tc(const Mechanism& m, const EmitOptions& opt, const 
   const TcBasis& b = p.b;
   const int ns = m.ns, K = b.K, G = kGroups, RT = kRowsChunk / G, QW = K / (4 * G);   // QW: groups of four species per compute group
   const int kThreads = 128 * G + 64;
-  const bool visc = p.part == 1, mixed = p.mixed;
+  const bool visc = p.part == 1, diff = p.part == 2, thermo = p.part == 3, mixed = p.mixed;
   const int NST = (int)p.st.size();
   std::ostringstream s;
   s << "// mechanism " << m.name << ": " << m.ns << " species, " << m.nr() << " reactions\n";
@@ -555,7 +580,7 @@ std::string emit_transport_tc(const Mechanism& m, const EmitOptions& opt, const 
   const int rpad = p.chunks * kRowsChunk;
   std::vector<double> rs(rpad, 0.0);
   for (int r = b.first; r < b.rows; ++r)
-    rs[r] = visc ? std::ldexp(1.0 / m.W[r - b.first], 18 - b.rho[r]) : std::ldexp(1.0, b.rho[0] - b.rho[r]);
+    rs[r] = thermo ? std::ldexp(1.0, b.rho[r]) : visc ? std::ldexp(1.0 / m.W[r - b.first], 18 - b.rho[r]) : std::ldexp(1.0, b.rho[0] - b.rho[r]);
   s << "__device__ const float2 kx_rs[" << rpad << "] = {" << list(rs, true) << "};\n";
   // basis functions
   s << "__device__ const float2 kx_phi[" << 32 * (b.M + 1) << "] = {";
@@ -569,15 +594,15 @@ std::string emit_transport_tc(const Mechanism& m, const EmitOptions& opt, const 
     << list(std::vector<double>(b.g1, b.g1 + 5), true) << "};\n";
   s << "extern \"C\" __global__ void __launch_bounds__(" << kThreads << ", 1) " << entry
     << "(const double* __restrict__ T_, const double* __restrict__ P_, const double* __restrict__ Y_, long long ld, "
-    << "double* __restrict__ out0_, double* __restrict__ out1_, double* __restrict__ out2_, long long n)\n{\n";
+    << "double* __restrict__ out0_, double* __restrict__ out1_, " << (thermo ? "" : "double* __restrict__ out2_, ") << "long long n)\n{\n";
   s << "  __shared__ __align__(8) unsigned long long bars[" << 2 * p.slots + 5 << "];\n";
   s << "  __shared__ unsigned tmem_addr;\n";
   s << "  kx_load_tables();\n";
   s << "  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;\n";
   s << "  unsigned char* const slots = kx_dyn;\n";
   s << fmt("  float2* const sphi = (float2*)(kx_dyn + %d);\n", p.slots * p.slot_bytes);
-  s << fmt("  float2* const sred = sphi + %d;   // [24][128]: values exchanged between the compute groups\n", (b.M + 1) * kStates);
-  s << fmt("  float2* const sph = sred + %d;    // basis polynomials\n", 24 * kStates);
+  s << fmt("  float2* const sred = sphi + %d;   // [][128]: values exchanged between the compute groups\n", (b.M + 1) * kStates);
+  s << fmt("  float2* const sph = sred + %d;    // basis polynomials\n", p.red * kStates);
   s << fmt("  float2* const srs = sph + %d;    // row scales\n", 32 * (b.M + 1));
   s << fmt("  int* const sec = (int*)(srs + %d);   // column exponents\n", rpad);
   const bool stage_y = K <= 64;
@@ -669,7 +694,7 @@ std::string emit_transport_tc(const Mechanism& m, const EmitOptions& opt, const 
   s << "    for (long long t = blockIdx.x; t < tiles; t += gridDim.x) {\n"
     << "      const bool in = t * 128 + s < n;\n"
     << "      bool bad = !(T > 0.0 && P > 0.0 && T < KX_INF && P < KX_INF);\n"
-    << "      bool gen = !(T >= " << D(kTcTlo) << " && T <= " << D(kTcThi) << ");\n";
+    << (thermo ? std::string("      bool gen = false;\n") : fmt("      bool gen = !(T >= %s && T <= %s);\n", D(kTcTlo).c_str(), D(kTcThi).c_str()));
   auto yval = [&](const std::string& j) {
     return stage_y ? fmt("sy[(%s) * 128 + s]", j.c_str()) : fmt("((%s) < %d ? Y_[(long long)(%s) * ld + i] : 0.0)", j.c_str(), ns, j.c_str());
   };
@@ -737,6 +762,7 @@ std::string emit_transport_tc(const Mechanism& m, const EmitOptions& opt, const 
   s << "      const long long in1 = min((t + gridDim.x) * 128 + s, n - 1);\n"
     << "      const double T1 = T_[in1], P1 = P_[in1];\n";
   if (stage_y) copy_y("      ", "in1");
+  if (!thermo) {
   // ln T and the basis functions, dealt to the groups, while the first matrix products run
   s << "      const kx_df L = kx_df_log(kx_df_mul(kx_d2df_i(gen ? 1000.0 : T), " << DFc(1.0 / kTcTmid) << "));   // ln T - L_mid\n"
     << "      const kx_df tb = kx_df_mul(L, " << DFc(1.0 / kTcLhalf) << "), t2 = kx_df_mul(tb, tb);\n";
@@ -795,13 +821,15 @@ std::string emit_transport_tc(const Mechanism& m, const EmitOptions& opt, const 
     }
   }
   s << "      KX_COMPUTE_SYNC;\n";
+  }
   // rows
   if (visc) s << "      kx_df mu = kx_mk(0.0f, 0.0f);\n";
-  s << (mixed ? "      float fac = 0.0f, sYs = 0.0f;\n" : "      kx_df fac = kx_mk(0.0f, 0.0f), sYs = fac;\n");
+  if (diff) s << (mixed ? "      float fac = 0.0f, sYs = 0.0f;\n" : "      kx_df fac = kx_mk(0.0f, 0.0f), sYs = fac;\n");
   s << "      for (int c = 0; c < " << p.chunks << "; c = c == 0 ? cnext : c + gy) {\n"
     << (mixed ? fmt("      float hi[%d];\n", RT) : fmt("      float hi[%d], lo[%d], sm[%d];\n", RT, RT, RT))
-    << fmt("      double yr[%d];\n", RT)
-    << fmt("      #pragma unroll\n      for (int a = 0; a < %d; ++a) {\n", RT)
+    << (thermo ? std::string() : fmt("      double yr[%d];\n", RT));
+  if (!thermo)
+    s << fmt("      #pragma unroll\n      for (int a = 0; a < %d; ++a) {\n", RT)
     << fmt("        const int k = c * 16 + wg * %d + a - %d;\n", RT, b.first)
     << fmt("        yr[a] = k >= 0 && k < %d ? Y_[(long long)k * ld + i] : 0.0;\n      }\n", ns);
   for (int st = 0; st < NST; ++st) {
@@ -816,12 +844,42 @@ std::string emit_transport_tc(const Mechanism& m, const EmitOptions& opt, const 
     s << fmt("      #pragma unroll\n      for (int a = 0; a < %d; ++a)", RT) << " { const kx_df w = kx_ts(hi[a], sm[a]); const kx_df z = kx_ts(w.hi, __fadd_rn(w.lo, lo[a])); hi[a] = z.hi; lo[a] = z.lo; }\n";
   }
   const char* LO = mixed ? "0.0f" : "lo[a]";
+  if (thermo) {
+    s << fmt("      #pragma unroll\n      for (int a = 0; a < %d; ++a) sred[(8 + c * 16 + wg * %d + a) * 128 + s] = make_float2(hi[a], lo[a]);\n      }\n", RT, RT)
+      << "      KX_COMPUTE_SYNC;\n"
+      // c_p = sum B_n x^n, h = h(x = 0) + T_half x sum B_n/(n + 1) x^n over the T_mid groups
+      << "      if (wg < 2 && in && !bad && !gen) {\n"
+      << "        const kx_df Td = kx_d2df_i(T);\n        kx_df v = kx_mk(0.0f, 0.0f);\n";
+    for (size_t g = 0; g < p.mids.size(); ++g) {
+      long long bits;
+      std::memcpy(&bits, &p.mids[g], 8);
+      s << fmt("        {\n          const bool low = __double_as_longlong(T) < %lldLL;\n", bits)
+        << fmt("          const kx_df xc = kx_df_add(Td, kx_mk(low ? %s : %s, 0.0f));\n", F(-kThTc[0]).c_str(), F(-kThTc[1]).c_str())
+        << fmt("          const float xs = low ? %s : %s;\n", F(1.0 / kThHalf[0]).c_str(), F(1.0 / kThHalf[1]).c_str())
+        << "          const kx_df x = kx_mk(xc.hi * xs, xc.lo * xs);\n"
+        << fmt("          const int r0 = low ? %d : %d;\n", 12 * (int)g, 12 * (int)g + 6)
+        << "          kx_df B[6];\n          #pragma unroll\n          for (int k = 0; k < 6; ++k) {\n"
+        << "            const float2 q = sred[(8 + r0 + k) * 128 + s]; const float f = srs[r0 + k].x;\n"
+        << "            B[k] = kx_mk(q.x * f, q.y * f);\n          }\n"
+        << "          if (wg == 0) {\n"
+        << "            v = kx_df_add(v, kx_df_fma(kx_df_fma(kx_df_fma(kx_df_fma(B[4], x, B[3]), x, B[2]), x, B[1]), x, B[0]));\n"
+        << "          } else {\n"
+        << fmt("            kx_df q = kx_df_mul(B[4], %s);\n", DFc(0.2).c_str())
+        << fmt("            q = kx_df_fma(q, x, kx_df_mul(B[3], %s));\n", DFc(0.25).c_str())
+        << fmt("            q = kx_df_fma(q, x, kx_df_mul(B[2], %s));\n", DFc(1.0 / 3.0).c_str())
+        << fmt("            q = kx_df_fma(q, x, kx_df_mul(B[1], %s));\n", DFc(0.5).c_str())
+        << "            q = kx_df_fma(q, x, B[0]);\n"
+        << "            v = kx_df_add(v, kx_df_fma(q, xc, B[5]));\n"
+        << "          }\n        }\n";
+    }
+    s << "        (wg == 0 ? out0_ : out1_)[i] = kx_df2d_s(v, -18 - sc);\n      }\n";
+  } else {
   s << "      if (c == 0) {\n"
     << fmt("        #pragma unroll\n        for (int a = 0; a < %d; ++a)\n          if (wg * %d + a < %d) sred[(8 + wg * %d + a) * 128 + s] = make_float2(hi[a], %s);\n", RT, RT, b.first, RT, LO)
     << "        KX_COMPUTE_SYNC;\n"
     << "        const float2 c0 = sred[8 * 128 + s], c1 = sred[9 * 128 + s], g0 = sred[4 * 128 + s];\n"
     << "        if (!gen && !(c0.x > 0.0f)) bad = true;\n";
-  if (!visc) {
+  if (diff) {
     // D_k = (1 - Y_k/sum Y) (p_atm/p) sigma / sum_{j != k} (Y_j/W_j)/D_kj
     if (!mixed)
       s << "        sYs = kx_mk(c1.x, c1.y);\n"
@@ -906,20 +964,24 @@ std::string emit_transport_tc(const Mechanism& m, const EmitOptions& opt, const 
         << "        out0_[i] = kx_f2d(mu.hi * g0.x);\n";
     s << "      }\n";
   }
+  }
   // states outside the domain, outside the basis' temperatures or with non-finite mass fractions
   s << "      if (cy == 0 && __any_sync(0xffffffffu, in && (bad || gen || !ok))) {\n"
-    << "        double isig = 0.0;\n"
-    << "        if (!bad && ok) {\n"
-    << "          double sy = 0.0;\n"
-    << fmt("          for (int j = 0; j < %d; ++j) sy = fma(Y_[(long long)j * ld + i], kx_iw[j], sy);\n", ns)
-    << "          isig = 1.0 / sy;\n"
-    << "          if (!(isig > 0.0 && isig < KX_INF)) bad = true;\n"
-    << "        }\n"
-    << "        bad = bad || !ok;\n"
-    << "        if (in && bad) {\n"
+    << "        bad = bad || !ok;\n";
+  if (!thermo)
+    s << "        double isig = 0.0;\n"
+      << "        if (!bad) {\n"
+      << "          double sy = 0.0;\n"
+      << fmt("          for (int j = 0; j < %d; ++j) sy = fma(Y_[(long long)j * ld + i], kx_iw[j], sy);\n", ns)
+      << "          isig = 1.0 / sy;\n"
+      << "          if (!(isig > 0.0 && isig < KX_INF)) bad = true;\n"
+      << "        }\n";
+  s << "        if (in && bad) {\n"
     << "          if (wg == 0) atomicMin(&kx_bad_first, (unsigned long long)i);\n";
-  if (visc) s << "          if (wg == 0) { out0_[i] = KX_NAN; out1_[i] = KX_NAN; }\n        } else if (in && gen && wg == 0) {\n"
-              << "          const double2 v = kx_visc_state(Y_, ld, i, kx_d2df(log(T) - " << D(kTcLmid) << "), isig);\n          out0_[i] = v.x; out1_[i] = v.y;\n        }\n";
+  if (!diff) s << "          if (wg == 0) { out0_[i] = KX_NAN; out1_[i] = KX_NAN; }\n        } else if (in && gen && wg == 0) {\n"
+               << (visc ? fmt("          const double2 v = kx_visc_state(Y_, ld, i, kx_d2df(log(T) - %s), isig);\n", D(kTcLmid).c_str())
+                        : std::string("          const double2 v = kx_thermo_state(Y_, ld, i, T);\n"))
+               << "          out0_[i] = v.x; out1_[i] = v.y;\n        }\n";
   else s << fmt("          for (int k = wg; k < %d; k += %d) out2_[(long long)k * ld + i] = KX_NAN;\n        }\n", ns, G)
          << "        const kx_df Lt = kx_d2df(log(gen && !bad ? T : 1000.0) - " << D(kTcLmid) << ");\n"
          << "        for (unsigned w = __ballot_sync(0xffffffffu, in && gen && !bad); w; w &= w - 1) {\n"
@@ -938,14 +1000,14 @@ std::string emit_transport_tc(const Mechanism& m, const EmitOptions& opt, const 
     for (int q = 1; q <= b.M; ++q) f += b.phi[q].size() * ((mixed || b.E[q] <= kPhiE) ? 2.0 : 12.0);
     double per = mixed ? 10 : 45;
     for (int q = 0; q <= b.M; ++q) per += (mixed || b.E[q] <= kFloatE) ? p.lev[q] : (6 + 2 + (p.lev[q] >= 3 ? 5 : 0) + (p.lev[q] >= 4 ? 2 : 0) + (q ? 9 : 0));
-    counts->fp32 += f + per * ns;
-    counts->fp64 += visc ? 3 : ns + 1;
+    counts->fp32 += f + per * b.rows;
+    counts->fp64 += diff ? 1 : 3;
   }
   if (shape) {
     shape->threads = kThreads;
     shape->smem = p.smem;
     shape->states_per_block = kStates;
-    shape->row_chunks = visc ? 1 : p.chunks;
+    shape->row_chunks = diff ? p.chunks : 1;
   }
   return s.str();
 }

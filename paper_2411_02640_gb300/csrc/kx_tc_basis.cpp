@@ -333,4 +333,63 @@ bool tc_basis(const Mechanism& m, int part, bool mixed, TcBasis& b) {
   return true;
 }
 
+bool tc_thermo(const Mechanism& m, TcBasis& b, std::vector<double>& mids) {
+  const int ns = m.ns;
+  b = TcBasis();
+  b.ns = ns;
+  b.K = (ns + 15) / 16 * 16;
+  mids = m.Tmid;
+  std::sort(mids.begin(), mids.end());
+  mids.erase(std::unique(mids.begin(), mids.end()), mids.end());
+  if (mids.size() > 4) return false;
+  b.rows = 12 * (int)mids.size();
+  b.E.assign(1, 0);
+  b.phi.assign(1, std::vector<double>(1, 1.0));
+  b.cheb = b.phi;
+  b.ecol.assign(ns, 0);
+  double wmin = m.W[0];
+  for (double w : m.W) wmin = std::min(wmin, w);
+  for (int k = 0; k < ns; ++k) {
+    int e;
+    std::frexp(wmin / m.W[k], &e);
+    b.ecol[k] = std::min(0, e);
+    if (b.ecol[k] < -40) return false;
+  }
+  std::vector<double> f((size_t)b.rows * ns, 0.0);
+  for (int k = 0; k < ns; ++k) {
+    const int g = (int)(std::lower_bound(mids.begin(), mids.end(), m.Tmid[k]) - mids.begin());
+    for (int rg = 0; rg < 2; ++rg) {
+      const double* a = rg == 0 ? &m.a_lo[7 * k] : &m.a_hi[7 * k];
+      double d[5];
+      shift_poly(a, kThTc[rg], 1.0, d);
+      HostDD h = {a[5], 0.0}, t = {kThTc[rg], 0.0};
+      for (int n = 0; n < 5; ++n) {
+        const HostDD q = hdd_mul({a[n], 0.0}, t);
+        const double v = q.hi / (n + 1), r = std::fma(-v, (double)(n + 1), q.hi) + q.lo;
+        h = hdd_add(h, hdd_norm(v, r / (n + 1)));
+        t = hdd_mul(t, {kThTc[rg], 0.0});
+      }
+      double p = 1.0;
+      for (int n = 0; n < 5; ++n, p *= kThHalf[rg]) f[(size_t)(12 * g + 6 * rg + n) * ns + k] = d[n] * p * (R_U / m.W[k]);
+      f[(size_t)(12 * g + 6 * rg + 5) * ns + k] = (h.hi + h.lo) * (R_U / m.W[k]);
+    }
+  }
+  b.rho.assign(b.rows, 0);
+  b.coef.assign(f.size(), 0.0);
+  for (int r = 0; r < b.rows; ++r) {
+    double mx = 0;
+    for (int k = 0; k < ns; ++k) {
+      const double v = std::ldexp(f[(size_t)r * ns + k], -b.ecol[k]);
+      if (!std::isfinite(v)) return false;
+      mx = std::max(mx, std::fabs(v));
+    }
+    int e = 0;
+    if (mx > 0) std::frexp(mx, &e);
+    if (e > 100 || e < -100) return false;
+    b.rho[r] = e;
+    for (int k = 0; k < ns; ++k) b.coef[(size_t)r * ns + k] = std::ldexp(f[(size_t)r * ns + k], -b.ecol[k] - e);
+  }
+  return true;
+}
+
 }  // namespace kx

@@ -30,4 +30,10 @@ struct TcBasis {
 
 bool tc_basis(const Mechanism& m, int part, bool mixed, TcBasis& b);
 
+// Thermo: the NASA-7 blocks are polynomials in T, so their basis is exact: for every distinct T_mid and
+// range six rows, R_U/W_j times the coefficients of c_p/R in x = (T - kThTc)/kThHalf (x^0 .. x^4) and
+// H/R at x = 0; rows 12 g + 6 (T >= T_mid) + 0 .. 5, M = 0.  mids receives the distinct T_mid.
+constexpr double kThTc[2] = {600.0, 2048.0}, kThHalf[2] = {512.0, 2048.0};
+bool tc_thermo(const Mechanism& m, TcBasis& b, std::vector<double>& mids);
+
 }  // namespace kx
