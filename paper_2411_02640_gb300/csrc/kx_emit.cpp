@@ -1692,11 +1692,22 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
   // mixed precision: float32 rates, float-pair chemical potentials and Gibbs sums, float64 accumulation
   const bool mx = opt.mixed;
   std::vector<DfClass> cls = emit_class_tables(g, m);
+  // With the float32 path for negligible reactions (most of them), large mechanisms' species vectors hold
+  // their two high parts first, and that path touches only those and the low parts of the accumulators: 8 and
+  // 4 + 4 bytes per entry instead of 16 and 8 + 8, and forms [X] in float32.  The kernel is bound by the traffic
+  // of these vectors (160/900: 6.4 KB a state), far beyond the L1 cache: 200003 states 5.39 -> 4.40 ms, and
+  // 3.75 at 80 registers.  53/325 gained nothing from it (traffic from L2 halved, 18 % fewer instructions, the
+  // float-pair path's own loads no longer ahead of time: 5.41 -> 5.60 ms) and keeps the full loads.
+  const bool lean = !rop && !mx && opt.rates_negligible == 0 && bounded;
 
   // ---- per state: T, ln T, 1/T, C_M, sigma, and the species vectors
   bool any_plog = false;
   for (auto& r : m.rx) any_plog |= r.kind == Kind::Plog;
   o("#define KX_PF(p) kx_mk((p)[0], (p)[1])");
+  if (lean) {
+    o("#define KX_SVH(k) (*(const float2*)&sv[k])          // {ln |C_k|, mu_k} high parts");
+    o("#define KX_SVL(k) (*((const float2*)&sv[k] + 1))    // low parts");
+  }
   o("const kx_df Td = kx_d2df_i(T);");
   o("const kx_df lnT = kx_df_log_d(T);");
   o("const kx_df iT = kx_df_div(kx_mk(1.0f, 0.0f), Td);");
@@ -1712,7 +1723,7 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
     o(fmt("float4 sv[%d];   // {ln |C_k|, C_k (float32), mu_k (pair)}", ns));
     if (!rop) o(fmt("double w[%d];", ns));
   } else {
-    o(fmt("float4 sv[%d];   // {ln |C_k| (pair), mu_k (pair)}", ns));
+    o(fmt("float4 sv[%d];   // {ln |C_k|, mu_k}: two pairs (with KX_SVH high parts first)", ns));
     if (!rop) o(fmt("kx_df w[%d];", ns));
   }
   o("kx_df sig = kx_mk(0.0f, 0.0f);");
@@ -1755,7 +1766,7 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
     o("  sv[k] = make_float4(l.hi, kx_df_mul(kx_d2df_i(Yk), KX_PF(kx_iwf + 2 * k)).hi * fC.hi, mk_.hi, mk_.lo);");
     if (!rop) o("  w[k] = 0.0;");
   } else {
-    o("  sv[k] = make_float4(l.hi, l.lo, mk_.hi, mk_.lo);");
+    o(lean ? "  sv[k] = make_float4(l.hi, mk_.hi, l.lo, mk_.lo);" : "  sv[k] = make_float4(l.hi, l.lo, mk_.hi, mk_.lo);");
     if (!rop) o("  w[k] = kx_mk(0.0f, 0.0f);");
   }
   o("}");
@@ -1779,12 +1790,18 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
     const int E = d.nre + d.npr, P = (E + 1 + 3) / 4 * 4;
     o(fmt("const int4* sp4 = (const int4*)kx_s%d;", ci));
     for (int q = 0; q < P / 4; ++q) o(fmt("int4 c%d = sp4[%d];", q, q));
-    for (int j = 0; j < E; ++j) o(fmt("float4 v%d = sv[%s];", j, spc("c", j).c_str()));
+    for (int j = 0; j < E; ++j) o(fmt(lean ? "float2 v%d = KX_SVH(%s);" : "float4 v%d = sv[%s];", j, spc("c", j).c_str()));
   };
   auto prefetch = [&](const DfClass& d) {
     const int E = d.nre + d.npr, P = (E + 1 + 3) / 4 * 4;
     for (int q = 0; q < P / 4; ++q) o(fmt("  const int4 n%d = sp4[%d * (r + 1) + %d];", q, P / 4, q));
-    for (int j = 0; j < E; ++j) o(fmt("  const float4 u%d = sv[%s];", j, spc("n", j).c_str()));
+    for (int j = 0; j < E; ++j) o(fmt(lean ? "  const float2 u%d = KX_SVH(%s);" : "  const float4 u%d = sv[%s];", j, spc("n", j).c_str()));
+  };
+  // the high and full values of entry j's ln |C| and mu
+  auto muh = [&](int j) { return fmt(lean ? "v%d.y" : "v%d.z", j); };
+  auto lnp = [&](int j) { return lean ? fmt("kx_mk(v%d.x, t%d.x)", j, j) : fmt("kx_mk(v%d.x, v%d.y)", j, j); };
+  auto mup = [&](int j, const char* sg) {
+    return lean ? fmt("kx_mk(%sv%d.y, %st%d.y)", sg, j, sg, j) : fmt("kx_mk(%sv%d.z, %sv%d.w)", sg, j, sg, j);
   };
   auto advance = [&](const DfClass& d) {
     const int E = d.nre + d.npr, P = (E + 1 + 3) / 4 * 4;
@@ -1835,8 +1852,8 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
       if (d.rev) {
         const int dn = d.npr - d.nre;
         std::string s = dn == 0 ? std::string("0.0f") : fmt("%s * lnPRTf", F(-dn).c_str());
-        for (int j = 0; j < d.nre; ++j) s += fmt(" - v%d.z", j);
-        for (int j = d.nre; j < d.nre + d.npr; ++j) s += fmt(" + v%d.z", j);
+        for (int j = 0; j < d.nre; ++j) s += " - " + muh(j);
+        for (int j = d.nre; j < d.nre + d.npr; ++j) s += " + " + muh(j);
         o("  b += fmaxf(" + s + ", 0.0f);");
       }
       o("  U = fmaxf(U, b);");
@@ -1877,12 +1894,13 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
         std::string pdecl = "int";
         for (int j = 0; j < E; ++j) pdecl += fmt("%s p%d = 0", j ? "," : "", j);
         o(pdecl + ";   // entries of the previous reaction (coefficient 0: nothing to add)");
-        o(mx ? "double qp = 0.0;" : "kx_df qp = kx_mk(0.0f, 0.0f);");
+        o(mx ? "double qp = 0.0;" : lean ? "float qp = 0.0f;" : "kx_df qp = kx_mk(0.0f, 0.0f);");
       }
       o("#pragma unroll 1");
       o(fmt("for (int r = 0; r < %d; ++r) {", (int)d.rx.size()));
       if (!rop)
-        for (int j = 0; j < E; ++j) o(fmt("  %s wl%d = w[p%d & 0xffff];", mx ? "const double" : "kx_df", j, j));
+        for (int j = 0; j < E; ++j)
+          o(lean ? fmt("  const float wl%d = w[p%d & 0xffff].lo;", j, j) : fmt("  %s wl%d = w[p%d & 0xffff];", mx ? "const double" : "kx_df", j, j));
       prefetch(d);
       for (int j = 0; j < E; ++j) o(fmt("  const int k%d = %s;", j, spc("c", j).c_str()));
       if (rop) o(fmt("  const int ri = %s;", comp("c", E).c_str()));
@@ -1891,9 +1909,7 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
       if (mx) {
         emit_class_mixed_body(o, d, (int)ci, E, c);
       } else {
-        if (tb) {
-          o(fmt("  const int2 e = kx_e%d[r];", (int)ci));
-          o("  const float4 f2 = f[2];");
+        auto third_body_df = [&]() {
           o("  kx_df X;   // [X] = eff_default C_M + (C_M/sigma) sum_e (eff_e - eff_default) Y_e/W_e");
           o("  if (e.y < 0) {");
           o("    const int kc = kx_effd[e.x].k;");
@@ -1907,6 +1923,29 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
           o("    X = kx_df_fma(kx_mk(f2.x, f2.y), cM, kx_df_mul(fC, t));");
           o("  }");
           c.fp32 += d.rx.size() * (kDfFma + kDfMul + 3 * (kDfFma + kDfMul + 12));
+        };
+        if (tb) {
+          o(fmt("  const int2 e = kx_e%d[r];", (int)ci));
+          o("  const float4 f2 = f[2];");
+          if (lean) {
+            // [X] in float32 from C = e^ln|C| (off by the logarithm's 4e-5, as the rates of this path are);
+            // the float-pair path forms its own
+            o("  float Xf = 0.0f;");
+            o("  if (e.y < 0) {");
+            o("    const int kc = kx_effd[e.x].k;");
+            o("    Xf = __expf(KX_SVH(kc).x);");
+            o("    if (anyneg && KX_NEG(kc)) Xf = -Xf;");
+            o("  } else {");
+            o("    for (int j = 0; j < e.y; ++j) {");
+            o("      const kx_effd_t q = kx_effd[e.x + j];");
+            o("      const float C = __expf(KX_SVH(q.k).x);");
+            o("      Xf = fmaf(q.ahi, anyneg && KX_NEG(q.k) ? -C : C, Xf);");
+            o("    }");
+            o("    Xf = fmaf(f2.x, cM.hi, Xf);");
+            o("  }");
+          } else {
+            third_body_df();
+          }
         }
         // Elementary and three-body reactions of a warp whose states all have this reaction's rate
         // below 2^-40 of their scale's anchor (2^(S+62), the largest rate so far; with the bounding
@@ -1922,7 +1961,7 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
             o("  const float4 f3 = f[3], f4 = f[4], f5 = f[5], f6 = f[6];");
             o("  float lfe = fmaf(f0.z, lnT.hi, fmaf(f1.x, iT.hi, f0.x));   // ln k_inf (float32)");
             o("  const float lk0e = fmaf(f3.x, lnT.hi, fmaf(f3.z, iT.hi, f2.z));   // ln k_0");
-            o("  const float lpe = lk0e - lfe + __logf(X.hi);   // ln Pr (nan for [X] < 0: no float32 path)");
+            o("  const float lpe = lk0e - lfe + __logf(Xf);   // ln Pr (nan for [X] < 0: no float32 path)");
             if (d.blend == Blend::Troe) {
               o("  const float lFc = __logf(f4.x * __expf(Td.hi * f5.x) + f4.z * __expf(Td.hi * f5.z) + __expf(f6.x * iT.hi)) * 0.434294482f;");
               o("  const float xe = fmaf(lpe, 0.434294482f, fmaf(-0.67f, lFc, -0.4f));");
@@ -1943,21 +1982,20 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
             o(d.kconst ? "  float lfe = f0.x;" : "  float lfe = fmaf(f0.z, lnT.hi, fmaf(f1.x, iT.hi, f0.x));   // ln |R_f| (float32)");
           }
           for (int j = 0; j < d.nre; ++j) o(fmt("  lfe += v%d.x;", j));
-          o(d.kind == Kind::ThreeBody ? "  const float lxe = __logf(X.hi);   // ln [X] (nan for [X] <= 0: no float32 path)"
+          o(d.kind == Kind::ThreeBody ? "  const float lxe = __logf(Xf);   // ln [X] (nan for [X] <= 0: no float32 path)"
                                       : "  const float lxe = 0.0f;");
           o("  float lme = lfe + lxe;");
           if (d.rev) {
             const int dn = d.npr - d.nre;
             std::string t = dn == 0 ? std::string("0.0f") : fmt("%s * lnPRT.hi", F(-dn).c_str());
-            for (int j = 0; j < d.nre; ++j) t += fmt(" - v%d.z", j);
-            for (int j = d.nre; j < E; ++j) t += fmt(" + v%d.z", j);
+            for (int j = 0; j < d.nre; ++j) t += " - " + muh(j);
+            for (int j = d.nre; j < E; ++j) t += " + " + muh(j);
             o("  const float lre = lfe + (" + t + ");   // ln |R_r| (float32)");
             o("  lme = fmaxf(lme, lre + lxe);");
           }
           std::string sfx = "0", srx = "0";
           for (int j = 0; j < d.nre; ++j) sfx += fmt(" ^ KX_NEG(k%d)", j);
           for (int j = d.nre; j < E; ++j) srx += fmt(" ^ KX_NEG(k%d)", j);
-          o("  kx_df q;");
           o("  if (__all_sync(__activemask(), lme < __fmul_rn(kx_i2f(S + 22), 0.693147182f))) {");
           o("    const float sl = __fmul_rn(kx_i2f(S), 0.693147182f);   // the rate scaled by 2^-S");
           o("    float qf = __expf(lfe - sl);");
@@ -1967,9 +2005,23 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
             o("    if (anyneg && (" + srx + ")) qr = -qr;");
             o("    qf -= qr;");
           }
-          o("    q = kx_mk(qf, 0.0f);");
+          if (d.kind == Kind::ThreeBody) o("    qf = __fmul_rn(qf, Xf);");
+          // the previous reaction's rate into the low parts of its accumulators (loaded at the top of this
+          // iteration): a float32 sum beside the float pairs' rounding errors, both far below 2^-40 of the
+          // largest rate
+          for (int j = 0; j < E; ++j)
+            o(fmt("    { const unsigned cj = (unsigned)p%d & 0xffff0000u; if (cj != 0u) w[p%d & 0xffff].lo = __fmaf_rn(__uint_as_float(cj), qp, wl%d); }", j, j, j));
+          o("    qp = qf;");
+          for (int j = 0; j < E; ++j) o(fmt("    p%d = %s;", j, comp("c", j).c_str()));
           o("  } else {");
-          c.fp32 += d.rx.size() * (6.0 + d.nre + (d.rev ? E + 3 : 0));
+          c.fp32 += d.rx.size() * (6.0 + 2.0 * d.nre + d.npr + (d.rev ? E + 3 : 0));
+        }
+        if (lean) {
+          if (!fastp) o("  {");
+          for (int j = 0; j < E; ++j)
+            o(fmt("  { const unsigned cj = (unsigned)p%d & 0xffff0000u; if (cj != 0u) w[p%d & 0xffff].lo = __fmaf_rn(__uint_as_float(cj), qp, wl%d); }", j, j, j));
+          for (int j = 0; j < E; ++j) o(fmt("  const float2 t%d = KX_SVL(k%d);", j, j));
+          if (tb) third_body_df();
         }
         o(d.kconst ? "  kx_df lk = kx_mk(f0.x, f0.y);   // k = A"
                    : "  kx_df lk = kx_df_fma_u(kx_mk(f0.z, f0.w), lnT, kx_df_fma_u(kx_mk(f1.x, f1.y), iT, kx_mk(f0.x, f0.y)));");
@@ -2019,7 +2071,7 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
         }
         // ln |R_f| (scaled by 2^-S) and the sign of prod C^nu'
         o("  kx_df lf = lk;");
-        for (int j = 0; j < d.nre; ++j) o(fmt("  lf = kx_df_add_u(lf, kx_mk(v%d.x, v%d.y));", j, j));
+        for (int j = 0; j < d.nre; ++j) o("  lf = kx_df_add_u(lf, " + lnp(j) + ");");
         std::string sfx = "0", srx = "0";
         for (int j = 0; j < d.nre; ++j) sfx += fmt(" ^ KX_NEG(k%d)", j);
         for (int j = d.nre; j < E; ++j) srx += fmt(" ^ KX_NEG(k%d)", j);
@@ -2030,10 +2082,8 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
         if (d.rev) {
           const int dn = d.npr - d.nre;
           o("  {   // ln(|R_r|/|R_f|) = sum nu mu - dn ln(p_atm/(R T))");
-          std::string first = d.nre > 0 ? "kx_df_neg(kx_mk(v0.z, v0.w))" : "kx_mk(v0.z, v0.w)";
-          o("    kx_df dl = " + first + ";");
-          for (int j = 1; j < E; ++j)
-            o(fmt("    dl = kx_df_add_u(dl, kx_mk(%sv%d.z, %sv%d.w));", j < d.nre ? "-" : "", j, j < d.nre ? "-" : "", j));
+          o("    kx_df dl = " + (d.nre > 0 ? "kx_df_neg(" + mup(0, "") + ")" : mup(0, "")) + ";");
+          for (int j = 1; j < E; ++j) o("    dl = kx_df_add_u(dl, " + mup(j, j < d.nre ? "-" : "") + ");");
           if (dn == 1 || dn == -1) o(fmt("    dl = kx_df_add_u(dl, %s);", dn == 1 ? "kx_df_neg(lnPRT)" : "lnPRT"));
           else if (dn != 0) o(fmt("    dl = kx_df_add_u(dl, kx_df_mulf(lnPRT, %s));", F(-dn).c_str()));
           o("    const int sr = anyneg ? (" + srx + ") : 0;");
@@ -2053,7 +2103,7 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
           o("  kx_df q = kx_df_mul_u(kx_df_exp_sc(L, Sr, __fmul_rn(kx_i2f(Sr), 0.693147182f)), fac);");
           c.fp32 += d.rx.size() * 4;
         } else {
-          const std::string qd = fastp ? "q" : "kx_df q";
+          const std::string qd = "kx_df q";
           if (bounded) {
             o("  " + qd + " = kx_df_mul_u(kx_df_exp_sc(L, S, lnSf), fac);   // |R| 2^-S (the products and sums after it take hi + lo as is)");
           } else {
@@ -2065,9 +2115,11 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
           o("    const int d = S - (ex - 62), d1 = max(d, -126), d2 = d - d1;");
           o("    const float f1 = __int_as_float((d1 + 127) << 23), f2 = d2 >= -126 ? __int_as_float((d2 + 127) << 23) : 0.0f;");
           o(fmt("    for (int k = 0; k < %d; ++k) w[k] = kx_mk(__fmul_rn(__fmul_rn(w[k].hi, f1), f2), __fmul_rn(__fmul_rn(w[k].lo, f1), f2));", ns));
-          for (int j = 0; j < E; ++j)
-            o(fmt("    wl%d = kx_mk(__fmul_rn(__fmul_rn(wl%d.hi, f1), f2), __fmul_rn(__fmul_rn(wl%d.lo, f1), f2));", j, j, j));
-          o("    qp = kx_mk(__fmul_rn(__fmul_rn(qp.hi, f1), f2), __fmul_rn(__fmul_rn(qp.lo, f1), f2));");
+          if (!lean) {
+            for (int j = 0; j < E; ++j)
+              o(fmt("    wl%d = kx_mk(__fmul_rn(__fmul_rn(wl%d.hi, f1), f2), __fmul_rn(__fmul_rn(wl%d.lo, f1), f2));", j, j, j));
+            o("    qp = kx_mk(__fmul_rn(__fmul_rn(qp.hi, f1), f2), __fmul_rn(__fmul_rn(qp.lo, f1), f2));");
+          }
           o("    S = ex - 62;");
           o("  }");
           o("  { const int d = ex - S; const float sc = d >= -126 ? __int_as_float((d + 127) << 23) : 0.0f; "
@@ -2075,8 +2127,16 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
           }
         }
         o("  if (sf) q = kx_df_neg(q);");
-        if (fastp) o("  }");
         if (d.kind == Kind::ThreeBody) { o("  q = kx_df_mul_u(q, X);"); c.fp32 += d.rx.size() * kDfMul; }
+        if (lean) {
+          // this rate into its accumulators at once; nothing stays pending
+          for (int j = 0; j < E; ++j)
+            o(fmt("  { const unsigned cj = (unsigned)%s & 0xffff0000u; if (cj != 0u) w[k%d] = kx_df_add_u(w[k%d], %s(q, __uint_as_float(cj))); p%d = 0; }",
+                  comp("c", j).c_str(), j, j, d.maxnu <= 2 ? "kx_df_scale2" : "kx_df_mulf", j));
+          o("  qp = 0.0f;");
+          o("  }");
+          c.fp32 += d.rx.size() * E * (kDfAdd + kDfMulf) / 2.0;
+        }
       }
       if (rop) {
         o(mx ? "  out_[(long long)ri * ld + i] = q;" : "  out_[(long long)ri * ld + i] = kx_df2d_s(q, Sr);");
@@ -2087,7 +2147,7 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
         o("  qp = q;");
         for (int j = 0; j < E; ++j) o(fmt("  p%d = %s;", j, comp("c", j).c_str()));
         c.fp64 += d.rx.size() * E;
-      } else {
+      } else if (!lean) {
         // the previous reaction's rate into its accumulators (loaded at the top of this iteration)
         for (int j = 0; j < E; ++j)
           o(fmt("  { const unsigned cj = (unsigned)p%d & 0xffff0000u; if (cj != 0u) w[p%d & 0xffff] = kx_df_add_u(wl%d, %s(qp, __uint_as_float(cj))); }",
@@ -2102,6 +2162,9 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
         for (int j = 0; j < E; ++j)
           o(fmt("{ const unsigned cj = (unsigned)p%d & 0xffff0000u; if (cj != 0u) { const int kk = p%d & 0xffff; w[kk] = fma(kx_f2d(__uint_as_float(cj)), qp, w[kk]); } }",
                 j, j));
+      else if (lean)
+        for (int j = 0; j < E; ++j)
+          o(fmt("{ const unsigned cj = (unsigned)p%d & 0xffff0000u; if (cj != 0u) { float* a = &w[p%d & 0xffff].lo; *a = __fmaf_rn(__uint_as_float(cj), qp, *a); } }", j, j));
       else if (!rop)
         for (int j = 0; j < E; ++j)
           o(fmt("{ const unsigned cj = (unsigned)p%d & 0xffff0000u; if (cj != 0u) { const int kk = p%d & 0xffff; w[kk] = kx_df_add_u(w[kk], %s(qp, __uint_as_float(cj))); } }",
@@ -4419,7 +4482,9 @@ std::string emit_kernel(const Mechanism& m, KernelKind kind, const EmitOptions& 
   const bool unrolled_rates = (kind == KernelKind::Wdot || kind == KernelKind::Rop) && !df_rates &&
                               !(opt.rates_mode == 2 || (opt.rates_mode == 0 && (m.ns > 64 || m.nr() > 400)));
   if (rreg == 0 && unrolled_rates) rreg = opt.mixed ? 96 : 128;
-  if (rreg == 0 && df_rates) rreg = opt.mixed ? 72 : 128;
+  // (large mechanisms' float-pair rates: 80, with the float32 path's short vectors; 160/900, 200003 states:
+  // 3.77 ms against 4.40 at 128)
+  if (rreg == 0 && df_rates) rreg = opt.mixed ? 72 : (kind == KernelKind::Wdot && !opt.scratch && m.ns > 64 && opt.rates_negligible == 0) ? 80 : 128;
   if (rreg == 0 && kind == KernelKind::Transport)
     rreg = opt.tr_layout != 3 ? 128 : (!opt.mixed && opt.tr_mode == 0 && opt.part == 1 && opt.diff_mode != 2) ? 80 : 64;
   if (rreg == 0 && kind == KernelKind::Thermo) rreg = 48;
