@@ -1723,7 +1723,7 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
     o(fmt("float4 sv[%d];   // {ln |C_k|, C_k (float32), mu_k (pair)}", ns));
     if (!rop) o(fmt("double w[%d];", ns));
   } else {
-    o(fmt("float4 sv[%d];   // {ln |C_k|, mu_k}: two pairs (with KX_SVH high parts first)", ns));
+    o(fmt(lean ? "float4 sv[%d];   // {ln |C_k|, mu_k}: the high parts, then the low parts" : "float4 sv[%d];   // {ln |C_k| (pair), mu_k (pair)}", ns));
     if (!rop) o(fmt("kx_df w[%d];", ns));
   }
   o("kx_df sig = kx_mk(0.0f, 0.0f);");
@@ -1961,7 +1961,7 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
             o("  const float4 f3 = f[3], f4 = f[4], f5 = f[5], f6 = f[6];");
             o("  float lfe = fmaf(f0.z, lnT.hi, fmaf(f1.x, iT.hi, f0.x));   // ln k_inf (float32)");
             o("  const float lk0e = fmaf(f3.x, lnT.hi, fmaf(f3.z, iT.hi, f2.z));   // ln k_0");
-            o("  const float lpe = lk0e - lfe + __logf(Xf);   // ln Pr (nan for [X] < 0: no float32 path)");
+            o("  const float lpe = lk0e - lfe + __logf(" + std::string(lean ? "Xf" : "X.hi") + ");   // ln Pr (nan for [X] < 0: no float32 path)");
             if (d.blend == Blend::Troe) {
               o("  const float lFc = __logf(f4.x * __expf(Td.hi * f5.x) + f4.z * __expf(Td.hi * f5.z) + __expf(f6.x * iT.hi)) * 0.434294482f;");
               o("  const float xe = fmaf(lpe, 0.434294482f, fmaf(-0.67f, lFc, -0.4f));");
@@ -1982,7 +1982,7 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
             o(d.kconst ? "  float lfe = f0.x;" : "  float lfe = fmaf(f0.z, lnT.hi, fmaf(f1.x, iT.hi, f0.x));   // ln |R_f| (float32)");
           }
           for (int j = 0; j < d.nre; ++j) o(fmt("  lfe += v%d.x;", j));
-          o(d.kind == Kind::ThreeBody ? "  const float lxe = __logf(Xf);   // ln [X] (nan for [X] <= 0: no float32 path)"
+          o(d.kind == Kind::ThreeBody ? std::string("  const float lxe = __logf(") + std::string(lean ? "Xf" : "X.hi") + ");   // ln [X] (nan for [X] <= 0: no float32 path)"
                                       : "  const float lxe = 0.0f;");
           o("  float lme = lfe + lxe;");
           if (d.rev) {
@@ -1996,6 +1996,7 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
           std::string sfx = "0", srx = "0";
           for (int j = 0; j < d.nre; ++j) sfx += fmt(" ^ KX_NEG(k%d)", j);
           for (int j = d.nre; j < E; ++j) srx += fmt(" ^ KX_NEG(k%d)", j);
+          if (!lean) o("  kx_df q;");
           o("  if (__all_sync(__activemask(), lme < __fmul_rn(kx_i2f(S + 22), 0.693147182f))) {");
           o("    const float sl = __fmul_rn(kx_i2f(S), 0.693147182f);   // the rate scaled by 2^-S");
           o("    float qf = __expf(lfe - sl);");
@@ -2005,6 +2006,11 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
             o("    if (anyneg && (" + srx + ")) qr = -qr;");
             o("    qf -= qr;");
           }
+          if (!lean) {
+            o("    q = kx_mk(qf, 0.0f);");
+            o("  } else {");
+            c.fp32 += d.rx.size() * (6.0 + d.nre + (d.rev ? E + 3 : 0));
+          } else {
           if (d.kind == Kind::ThreeBody) o("    qf = __fmul_rn(qf, Xf);");
           // the previous reaction's rate into the low parts of its accumulators (loaded at the top of this
           // iteration): a float32 sum beside the float pairs' rounding errors, both far below 2^-40 of the
@@ -2015,6 +2021,7 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
           for (int j = 0; j < E; ++j) o(fmt("    p%d = %s;", j, comp("c", j).c_str()));
           o("  } else {");
           c.fp32 += d.rx.size() * (6.0 + 2.0 * d.nre + d.npr + (d.rev ? E + 3 : 0));
+          }
         }
         if (lean) {
           if (!fastp) o("  {");
@@ -2103,7 +2110,7 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
           o("  kx_df q = kx_df_mul_u(kx_df_exp_sc(L, Sr, __fmul_rn(kx_i2f(Sr), 0.693147182f)), fac);");
           c.fp32 += d.rx.size() * 4;
         } else {
-          const std::string qd = "kx_df q";
+          const std::string qd = fastp && !lean ? "q" : "kx_df q";
           if (bounded) {
             o("  " + qd + " = kx_df_mul_u(kx_df_exp_sc(L, S, lnSf), fac);   // |R| 2^-S (the products and sums after it take hi + lo as is)");
           } else {
@@ -2127,6 +2134,7 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
           }
         }
         o("  if (sf) q = kx_df_neg(q);");
+        if (fastp && !lean) o("  }");
         if (d.kind == Kind::ThreeBody) { o("  q = kx_df_mul_u(q, X);"); c.fp32 += d.rx.size() * kDfMul; }
         if (lean) {
           // this rate into its accumulators at once; nothing stays pending
