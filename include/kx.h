@@ -73,8 +73,8 @@ typedef enum {
                     float32's exponent range, run on the float32 pipe -- and
                     the production rates are formed in log space and
                     accumulated in float pairs under a per-state power-of-two
-                    scale, reactions negligible for every state of a warp in
-                    float32 (see kx_production_rates); kx_options.rates_arith
+                    scale, reactions negligible in their state in float32
+                    (see kx_production_rates); kx_options.rates_arith
                     = 1 selects native float64
                     production rates and rates of progress, tr_mode = 1
                     native float64 transport.  kx_thermo is always
@@ -120,12 +120,13 @@ typedef struct {
   int compile_only;   /* 1: emit and compile but do not load onto a device (no GPU needed);
                          launch calls on such a handle return KX_ERR_UNSUPPORTED */
   int rates_layout;   /* double-float KX_FP64 production rates: 0 (default) by batch size -- the
-                         warp-cooperative kernel for batches below min(C, 49152 u) states and the
-                         thread-per-state kernel from there on, C being the thread-per-state
-                         kernel's resident capacity (one wave of its blocks on every SM; ~78k
-                         states on GB300 at 128 threads per block) and u the share of lane slots
+                         warp-cooperative kernel for small batches and the thread-per-state kernel
+                         from min(C, 19000 u^0.75) states on (mechanisms of up to 64 species and
+                         400 reactions) or min(C, 49152 u) (larger ones), C being the
+                         thread-per-state kernel's resident capacity (one wave of its blocks on
+                         every SM; ~155k and ~97k states on GB300) and u the share of lane slots
                          the warp-cooperative class rounds fill (~0.2 for 9/21, ~0.9 for 53/325);
-                         the crossover measured on GB300;
+                         the crossovers measured on GB300;
                          1 always one thread per state (species vectors in local memory);
                          2 always warp-cooperative (the states of a warp share its lanes: the
                          reactions of each class dealt out as (state, reaction) pairs, species
@@ -150,8 +151,8 @@ typedef struct {
                          under 0 and are refused under 2).  The two agree to ~1e-10 of each
                          entry's term scale, not bit for bit. */
   int rates_negligible; /* double-float KX_FP64 production rates: 0 (default) a reaction whose rate
-                         is below 2^-40 of its state's largest, for every state of a warp, is
-                         evaluated in float32 (its error is far inside the per-point bar, but a
+                         is below 2^-40 of its state's largest (above 64 species or 400
+                         reactions: for every state of a warp) is evaluated in float32 (its error is far inside the per-point bar, but a
                          species all of whose reactions are that small gets wdot_k to ~1e-4 of
                          itself); 1 every reaction in float pairs (wdot_k to ~1e-11 of the
                          species' own gross rate, for the species within 1e-40 of their state's
@@ -174,13 +175,16 @@ kx_status kx_mechanism_info(kx_handle h, int* n_species, int* n_reactions, doubl
 /* Net production rates wdot[N_s][ld] (Sec. A.2: Eq. (arrhenius), third-body
  * and falloff modifiers Eq. (c_i) and (blend), Eq. (K_p), Eq. (r_i) and the
  * stoichiometric sum wdot_k = sum_i nu_ki R_i).  KX_FP64 with the default
- * double-float kernel evaluates a reaction in float32 when, for every state of
- * a warp (32 consecutive states), its rate is below 2^-40 of that state's
- * largest rate, where float32's error leaves the result far inside the
- * float64 bar: a state's results can therefore differ, within the bar (~1e-11
- * of the per-point scale), with the states it shares a warp with (a call on a
- * sub-range that does not start at a multiple of 32 states, or a batch mixed
- * with other states); the same batch gives the same bits.  A species that
+ * double-float kernel evaluates a reaction in float32 when its rate is below
+ * 2^-40 of its state's largest rate, where float32's error leaves the result
+ * far inside the float64 bar.  Mechanisms of up to 64 species and 400
+ * reactions decide this for each state by itself, unless a state of the warp
+ * (32 consecutive states) has a negative mass fraction; larger ones, and such
+ * warps, take float32 where it holds for every state of the warp: a state's
+ * results can therefore differ, within the bar (~1e-11 of the per-point
+ * scale), with the states it shares a warp with (a call on a sub-range that
+ * does not start at a multiple of 32 states, or a batch mixed with other
+ * states); the same batch gives the same bits.  A species that
  * only such reactions produce or consume gets its wdot_k to ~1e-4 of itself
  * (still ~1e-16 of the per-point scale); kx_options.rates_negligible = 1
  * evaluates every reaction in float pairs (for finite differences). */

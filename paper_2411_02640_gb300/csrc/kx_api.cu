@@ -433,6 +433,12 @@ kx_status kx_load_mechanism(const char* path, const kx_options* opt, kx_handle* 
       k->states_per_block = w.states_per_block;
       k->lane_use = w.lane_use;
     }
+    if (sp.kind == kx::KernelKind::Wdot && !wc_spec && k->eopt.rates_layout != 2 && (h->opt.rates_arith != 1 || k->eopt.scratch) &&
+        kx::rates_swept(h->m, k->eopt, false) && (!opt || opt->block == 0)) {
+      // the warps of a block share the sweep's instruction fetches (2^20 states of 53/325 at 64 registers: blocks of
+      // 128 3.59 ms, 256 2.57, 512 2.76, 1024 3.6)
+      k->eopt.block = 256;
+    }
     if (sp.kind == kx::KernelKind::Transport) {
       // species vectors staged in shared memory: as many threads as fit in ~216 KB, a multiple of 32
       k->eopt.tr_layout = h->opt.tr_layout == 0 ? 3 : h->opt.tr_layout;
@@ -524,9 +530,8 @@ int64_t small_batch_below(const Kernel& wc, double scale) {
 
 // The production-rate kernel for a batch of n states.  Small float64-accurate batches go to the
 // warp-cooperative kernel, whose warps share each state: the thread-per-state kernel would leave
-// SMs idle and take one state's whole latency.  The crossover, measured on GB300, sits near 48k
-// states times the lane use of the warp-cooperative class rounds (53/325: ~44k, 160/900: ~46k, 9/21
-// with its few reactions per class: ~11k), and never above the thread-per-state kernel's resident
+// SMs idle and take one state's whole latency.  The crossover, measured on GB300, grows with the lane
+// use of the warp-cooperative class rounds, and is never above the thread-per-state kernel's resident
 // capacity.
 kx_status wdot_kernel_for(kx_mech* h, int64_t n, kx_precision precision, const char** name) {
   *name = precision == KX_FP64 ? "wdot_fp64" : "wdot_mixed";
@@ -537,7 +542,10 @@ kx_status wdot_kernel_for(kx_mech* h, int64_t n, kx_precision precision, const c
   if (s == KX_OK) s = ensure_ready(h, *wc);
   if (s != KX_OK) return s;
   const int64_t cap = (int64_t)tps->max_blocks * tps->eopt.block;
-  if (n < std::min<int64_t>(cap, (int64_t)(49152.0 * wc->lane_use))) *name = "wdot_fp64_wc";
+  // the swept kernel (53/325: 154 us up to 16k states, 9/21: 26) against the warp-cooperative kernel's 8.4 and 4.2 us
+  // per 1024 states: crossovers at 17.5k (lane use 0.92) and 6k (0.22)
+  const double below = kx::rates_swept(h->m, tps->eopt, false) ? 19000.0 * std::pow(wc->lane_use, 0.75) : 49152.0 * wc->lane_use;
+  if (n < std::min<int64_t>(cap, (int64_t)below)) *name = "wdot_fp64_wc";
   return KX_OK;
 }
 

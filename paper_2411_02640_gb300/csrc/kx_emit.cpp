@@ -540,17 +540,27 @@ template <typename V> struct kx_strided {
 // nu q for a coefficient nu in {-2, -1, 1, 2}: an exact scaling of both parts
 // (larger coefficients take the float-pair product kx_df_mulf)
 __device__ __forceinline__ kx_df kx_df_scale2(kx_df q, float nu) { return kx_mk(__fmul_rn(q.hi, nu), __fmul_rn(q.lo, nu)); }
-// (a.hi + a.lo) 2^S as a double: one float64 addition, the power of two
-// added to the exponent field (ldexp only when the result leaves the normal
-// range)
+// (a.hi + a.lo) 2^S as a double, in integers (the float64 pipe takes 16
+// cycles of an SM per warp instruction), the power of two added to the
+// exponent field (ldexp only when the result leaves the normal range)
 __device__ __forceinline__ double kx_df2d_s(kx_df a, int S) {
   if (a.hi == 0.0f && a.lo == 0.0f) return 0.0;   // (an unnormalised sum may hold its value in lo alone)
   if (!(fabsf(a.hi) < KX_INF_F)) return (double)a.hi;
-  const double d = kx_f2d(a.hi) + kx_f2d(a.lo);
-  if (d == 0.0) return 0.0;
-  const int hi = __double2hiint(d);
-  const int E = ((hi >> 20) & 0x7ff) + S;
-  if (E > 0 && E < 0x7ff) return __hiloint2double(hi + (int)((unsigned)S << 20), __double2loint(d));
+  const kx_df s = kx_ts(a.hi, a.lo);
+  const int h = __float_as_int(s.hi), e = (h >> 23) & 0xff;
+  if (e < 64 || e > 253) {
+    const double d = (double)s.hi + (double)s.lo;
+    return ldexp(d, S);
+  }
+  // hi's 24 bits as the double's leading ones, lo in units of its last (2^(e - 52); of 2^(e - 53) where hi is a
+  // power of two that lo takes the difference below), rounded once: the sum's nearest double
+  const bool dn = (h & 0x7fffff) == 0 && ((h ^ __float_as_int(s.lo)) < 0);
+  const float u = __fmul_rn(__fmul_rn(s.lo, __int_as_float((254 - e) << 23)), dn ? 0x1p53f : 0x1p52f);
+  const int l = __float2int_rn(h < 0 ? -u : u);
+  long long b = (((long long)(h & 0x7fffffff) + (896LL << 23)) << 29) + l;
+  const int E = (int)(b >> 52) + S;
+  const double d = __longlong_as_double(b | ((long long)(h & 0x80000000) << 32));
+  if (E > 0 && E < 0x7ff) return __longlong_as_double(__double_as_longlong(d) + ((long long)S << 52));
   return ldexp(d, S);
 }
 // ln(1 + y) for 0 <= y <= 1 (absolute error about 1e-15)
@@ -1681,6 +1691,187 @@ std::vector<DfClass> emit_class_tables(Out& g, const Mechanism& m, bool merged =
   return cls;
 }
 
+// The float32 sweep.  Per state most reactions are negligible (98 % of (reaction, state) pairs of the 53/325
+// workload run below 2^-40 of the state's largest rate), and all that such a reaction needs is float32: about
+// 35 instructions when they are straight-line code with the reaction's constants as immediates and the sums in
+// registers, against 180 in a table-driven loop over local vectors (addresses, masks and moves).  Pass 1 bounds the state's rates (M, log2 of the largest);
+// pass 2 adds every reaction below 2^(M - 40) to the state's float32 sums, scaled by 2^-S, and marks the others
+// in a bit mask; the warp's marked reactions (any state's) become a list that the class loops then evaluate in
+// float pairs, each state taking those that it marked.  The choice is the state's own: its results do not
+// depend on the states beside it, but for a negative mass fraction among the warp's states (emit_rates_class_df).
+// 2^20 states: 53/325 5.35 -> 2.57 ms, of which the species' logarithms and Gibbs energies take 25 %, pass 1
+// 18 %, pass 2 37 %, the marked reactions (16 of 325 per warp, 7 per state) 15 %, the results 18 %; 47 % of the
+// issue slots, the rest waits on the per-thread vectors (1.7 KB a state, far beyond the L1 cache).
+void emit_sweep(Out& o, Out& g, const Mechanism& m, const std::vector<DfClass>& cls, const EmitOptions& opt, OpCounts& c) {
+  const int ns = m.ns, nr = m.nr();
+  const double L2E = 1.4426950408889634;
+  const int W = (nr + 31) / 32;
+  g("__device__ __forceinline__ float kx_ex2(float x) { float r; asm(\"ex2.approx.ftz.f32 %0, %1;\" : \"=f\"(r) : \"f\"(x)); return r; }");
+  g("__device__ __forceinline__ float kx_lg2(float x) { float r; asm(\"lg2.approx.ftz.f32 %0, %1;\" : \"=f\"(r) : \"f\"(x)); return r; }");
+  o("const bool run = !__any_sync(0xffffffffu, anyneg);   // no state of this warp has a negative mass fraction");
+  o("float tL = KX_L2(lnT.hi, lnT.lo), pL = KX_L2(lnPRT.hi, lnPRT.lo), iTf = iT.hi, Tf = Td.hi, cMf = cM.hi;");
+  o("float M = -1.0e30f;");
+  auto arr = [&](const Arrh& a) {   // log2 k
+    std::string t = F(std::log(a.A > 0 ? a.A : 1e-300) * L2E);
+    if (a.beta != 0.0) t = fmt("fmaf(%s, tL, %s)", F(a.beta).c_str(), t.c_str());
+    if (a.E != 0.0) t = fmt("fmaf(%s, iTf, %s)", F(-a.E * L2E).c_str(), t.c_str());
+    return t;
+  };
+  // float e = log2 |R_f|, r = log2 |R_r|
+  auto estimate = [&](const Reaction& r, bool bound) {
+    std::string t;
+    if (r.third_body()) {
+      std::string X;
+      if (r.collider >= 0) {
+        X = fmt("kx_ex2(h%d)", r.collider);
+      } else {
+        X = fmt("%s * cMf", F(r.default_eff).c_str());
+        for (auto& x : r.eff)
+          if (x.second != r.default_eff) X = fmt("fmaf(%s, kx_ex2(h%d), %s)", F(x.second - r.default_eff).c_str(), x.first, X.c_str());
+      }
+      t += "const float X = " + X + ", x = kx_lg2(X); ";
+    }
+    if (r.kind == Kind::Falloff || r.kind == Kind::ChemAct) {
+      t += "const float ki = " + arr(r.k) + ", k0 = " + arr(r.k0) + ", lp = k0 - ki + x; ";
+      if (r.blend == Blend::Troe) {
+        t += fmt("const float lc = kx_lg2(fmaf(%s, kx_ex2(Tf * %s), fmaf(%s, kx_ex2(Tf * %s), kx_ex2(iTf * %s)))) * 0.301029996f; ",
+                 F(1.0 - r.troe[0]).c_str(), F(-L2E / r.troe[1]).c_str(), F(r.troe[0]).c_str(), F(-L2E / r.troe[2]).c_str(),
+                 F(-r.troe[3] * L2E).c_str());
+        t += "const float xe = fmaf(lp, 0.301029996f, fmaf(-0.67f, lc, -0.4f)); "
+             "const float fe = __fdividef(xe, fmaf(-0.14f, xe, fmaf(-1.27f, lc, 0.75f))); "
+             "const float lF = __fdividef(3.32192809f * lc, fmaf(fe, fe, 1.0f)); ";
+      } else if (r.blend == Blend::Sri) {
+        t += fmt("const float lP = lp * 0.301029996f; const float lF = fmaf(%s, tL, %s) + __fdividef(kx_lg2(fmaf(%s, kx_ex2(iTf * %s), "
+                 "kx_ex2(Tf * %s))), fmaf(lP, lP, 1.0f)); ",
+                 F(r.sri[4]).c_str(), F(std::log(r.sri[3]) * L2E).c_str(), F(r.sri[0]).c_str(), F(-r.sri[1] * L2E).c_str(), F(-L2E / r.sri[2]).c_str());
+      } else {
+        t += "const float lF = 0.0f; ";
+      }
+      t += "const float l1 = kx_lg2(1.0f + kx_ex2(-fabsf(lp))); ";
+      t += r.kind == Kind::Falloff ? "float e = ki + (lp < 0.0f ? lp - l1 : -l1) + lF; " : "float e = k0 + lF - (lp < 0.0f ? l1 : lp + l1); ";
+    } else if (r.kind == Kind::Plog) {
+      if (!bound) return std::string();   // always marked
+      t += "float e, k1; e = k1 = " + arr(Arrh{r.plog[0][1], r.plog[0][2], r.plog[0][3]}) + "; ";
+      for (size_t j = 1; j < r.plog.size(); ++j) {   // between pressures j - 1 and j, or above j
+        const double l0 = std::log(r.plog[j - 1][0]), l1 = std::log(r.plog[j][0]);
+        t += fmt("{ const float t = fminf((lnP.hi - %s) * %s, 1.0f), k0 = k1; k1 = %s; if (t > 0.0f) e = fmaf(t, k1 - k0, k0); } ", F(l0).c_str(),
+                 F(1.0 / (l1 - l0)).c_str(), arr(Arrh{r.plog[j][1], r.plog[j][2], r.plog[j][3]}).c_str());
+      }
+    } else {
+      t += "float e = " + arr(r.k) + "; ";
+    }
+    t += "e = e";
+    for (int k : entries(r.reac)) t += fmt(" + h%d", k);
+    if (r.kind == Kind::ThreeBody) t += " + x";
+    t += "; ";
+    if (r.reversible) {
+      const int dn = sum_nu(r);
+      std::string d = dn == 0 ? std::string("e") : fmt("fmaf(%s, pL, e)", F(-dn).c_str());
+      const auto re = entries(r.reac), pr = entries(r.prod);
+      for (size_t j = 0; j < std::max(re.size(), pr.size()); ++j) {
+        std::string q;
+        if (j < pr.size()) q = fmt("u%d", pr[j]);
+        if (j < re.size()) q += fmt("%s u%d", q.empty() ? "-" : " -", re[j]);
+        d += " + (" + q + ")";
+      }
+      t += "const float r = " + d + "; ";
+    }
+    return t;
+  };
+  auto largest = [&](const Reaction& r) { return std::string(r.reversible ? "fmaxf(e, r)" : "e"); };
+  // Groups of reactions with a block barrier between them.  A warp on its own gets through straight-line code
+  // (about 350 KB for 325 reactions) at 10 cycles an instruction, the latency of fetching it; behind the barriers
+  // the warps of a block use what the first of them fetches, and the compiler cannot hold values across groups
+  // (in one basic block 3.6 KB of them spill), so each group reads its own species.  2^20 states of 53/325:
+  // without barriers 4.26 ms at 64 registers, 3.5 at 80; with them 2.57 (groups of 16; 8: 2.60, 12: 2.7, 32: 3.6)
+  const int GRP = 16;
+  int at = 0;
+  std::vector<int> order;
+  for (auto& d : cls) order.insert(order.end(), d.rx.begin(), d.rx.end());
+  auto loads = [&]() {
+    std::vector<char> need(ns, 0);
+    for (int q = at; q < std::min(nr, at + GRP); ++q) {
+      const Reaction& r = m.rx[order[q]];
+      for (auto& e : r.reac) need[e.first] |= r.reversible ? 3 : 1;
+      for (auto& e : r.prod) need[e.first] |= r.reversible ? 2 : 0;
+      for (auto& e : r.eff) need[e.first] |= 1;
+      if (r.collider >= 0) need[r.collider] |= 1;
+    }
+    for (int k = 0; k < ns; ++k) {
+      if (need[k] & 1) o(fmt("const float h%d = ((const volatile float2&)KX_HU(%d)).x;", k, k));
+      if (need[k] & 2) o(fmt("const float u%d = ((const volatile float2&)KX_HU(%d)).y;", k, k));
+    }
+  };
+  auto group = [&]() {
+    if (at % GRP == 0) {
+      o(fmt("%s__syncthreads(); if (run) {", at ? "} " : ""));
+      loads();
+    }
+    ++at;
+  };
+  o("// pass 1: the largest rate");
+  for (auto& d : cls)
+    for (int i : d.rx) group(), o("{ " + estimate(m.rx[i], true) + "M = fmaxf(M, " + largest(m.rx[i]) + "); }");
+  o("}");
+  o("// largest scaled rate near 2^63.5; |S| < 2^11 keeps S ln2 exact to the float-pair precision");
+  o("const int S = kx_rint(fminf(fmaxf(M, -1000.0f), 1000.0f)) - 63;");
+  o("const float lnSf = __fmul_rn(kx_i2f(S), 0.693147182f);   // S ln2 for the range tests of the scaled exponential");
+  o("const float Sf = kx_i2f(S), thr = M - 40.0f;");
+  // read back, so that the second pass forms its estimates again (the compiler would keep the first pass's)
+  o("volatile float back[5];");
+  o("back[0] = tL; back[1] = pL; back[2] = iTf; back[3] = Tf; back[4] = cMf;");
+  o("tL = back[0]; pL = back[1]; iTf = back[2]; Tf = back[3]; cMf = back[4];");
+  {
+    std::string a;
+    for (int k = 0; k < ns; ++k) a += fmt("%sa%d = 0.0f", k ? ", " : "float ", k);
+    o(a + ";");
+    o(fmt("__shared__ unsigned kx_msk[%d];", W * opt.block));
+    o("unsigned mw = 0u;   // marks of 32 reactions");
+  }
+  o("// pass 2: negligible reactions into the float32 sums, the others marked");
+  int bit = 0;
+  at = 0;
+  for (auto& d : cls)
+    for (int i : d.rx) {
+      group();
+      const Reaction& r = m.rx[i];
+      const std::string mark = fmt("mw |= 0x%xu;", 1u << (bit % 32));
+      ++bit;
+      const std::string put = bit % 32 && bit != nr ? std::string() : fmt(" kx_msk[%d + threadIdx.x] = mw; mw = 0u;", (bit - 1) / 32 * opt.block);
+      if (r.kind == Kind::Plog) { o(mark + put); continue; }
+      std::string t = "{ " + estimate(r, false);
+      t += "const bool p = " + largest(r) + " < thr; if (!p) " + mark + " ";
+      t += r.reversible ? "float q = kx_ex2(e - Sf) - kx_ex2(r - Sf); " : "float q = kx_ex2(e - Sf); ";
+      t += "q = p ? q : 0.0f;";
+      std::map<int, int> net;
+      for (auto& e : r.reac) net[e.first] -= e.second;
+      for (auto& e : r.prod) net[e.first] += e.second;
+      for (auto& kv : net) {
+        if (kv.second == 1) t += fmt(" a%d += q;", kv.first);
+        else if (kv.second == -1) t += fmt(" a%d -= q;", kv.first);
+        else if (kv.second != 0) t += fmt(" a%d = fmaf(%s, q, a%d);", kv.first, F(kv.second).c_str(), kv.first);
+      }
+      o(t + " }" + put);
+    }
+  o("}");
+  o("// the sums start the float-pair accumulators; the warp's list of marked reactions, in class order");
+  o("if (run) {");
+  for (int k = 0; k < ns; ++k) o(fmt("w[%d] = kx_mk(a%d, 0.0f);", k, k));
+  o("}");
+  o(fmt("__shared__ short kx_lst[%d];", opt.block / 32 * (nr + 2)));
+  o(fmt("short* const lst = kx_lst + (threadIdx.x >> 5) * %d;", nr + 2));
+  o("const bool lead = (threadIdx.x & 31) == 0;");
+  o("int cnt = 0;");
+  o("__syncwarp();");
+  for (int w = 0; w < W; ++w) {
+    o(fmt("for (unsigned a = __reduce_or_sync(0xffffffffu, run ? kx_msk[%d + threadIdx.x] : 0u); a; a &= a - 1) { if (lead) lst[cnt] = (short)(%d + __ffs(a) - 1); ++cnt; }", w * opt.block, 32 * w));
+  }
+  o("if (lead) lst[cnt] = 32767;");
+  o("__syncwarp();");
+  o("int pos = 0;");
+  c.fp32 += nr * 50.0;
+}
+
 void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& opt, bool rop, OpCounts& c) {
   const int ns = m.ns;
   // The per-state scale 2^-S of the accumulation: up to 64 species it is set by the first rate and
@@ -1699,6 +1890,9 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
   // 3.75 at 80 registers.  53/325 gained nothing from it (traffic from L2 halved, 18 % fewer instructions, the
   // float-pair path's own loads no longer ahead of time: 5.41 -> 5.60 ms) and keeps the full loads.
   const bool lean = !rop && !mx && opt.rates_negligible == 0 && bounded;
+  // Small mechanisms: a straight-line float32 sweep over all reactions first (emit_sweep), the class loops for
+  // those that it leaves
+  const bool sweep = rates_swept(m, opt, rop);
 
   // ---- per state: T, ln T, 1/T, C_M, sigma, and the species vectors
   bool any_plog = false;
@@ -1726,9 +1920,26 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
     o(fmt(lean ? "float4 sv[%d];   // {ln |C_k|, mu_k}: the high parts, then the low parts" : "float4 sv[%d];   // {ln |C_k| (pair), mu_k (pair)}", ns));
     if (!rop) o(fmt("kx_df w[%d];", ns));
   }
+  if (sweep) {
+    o("// the sweep's {log2 |C_k|, mu_k/ln 2}, each rounded to float32 once, until its sums take their place");
+    o("#define KX_HU(k) (*(float2*)&w[k])");
+    o("#define KX_L2(v, w) fmaf(v, 1.44269502f, fmaf(v, 1.92596303e-8f, (w) * 1.44269502f))");
+  }
   o("kx_df sig = kx_mk(0.0f, 0.0f);");
-  o(fmt("for (int k = 0; k < %d; ++k) sig = kx_df_fma(kx_d2df_i(Y_[(long long)k * ld + i]), KX_PF(kx_iwf + 2 * k), sig);", ns));
-  o("if (!(sig.hi > 0.0f && sig.hi < KX_INF_F)) KX_BAD_POINT");
+  if (sweep) {   // eight loads in flight: 28 instead of 66 thousand cycles of a warp's 800
+    o("#pragma unroll 1");
+    o(fmt("for (int k0 = 0; k0 < %d; k0 += 8) {", ns));
+    o("  double y8[8];");
+    o("#pragma unroll");
+    o(fmt("  for (int j = 0; j < 8; ++j) y8[j] = k0 + j < %d ? Y_[(long long)(k0 + j) * ld + i] : 0.0;", ns));
+    o("#pragma unroll");
+    o(fmt("  for (int j = 0; j < 8; ++j) sig = kx_df_fma(kx_d2df_i(y8[j]), KX_PF(kx_iwf + 2 * min(k0 + j, %d)), sig);", ns - 1));
+    o("}");
+  } else {
+    o(fmt("for (int k = 0; k < %d; ++k) sig = kx_df_fma(kx_d2df_i(Y_[(long long)k * ld + i]), KX_PF(kx_iwf + 2 * k), sig);", ns));
+  }
+  o(sweep ? "if (!(sig.hi > 0.0f && sig.hi < KX_INF_F)) { bad = true; sig = kx_mk(1.0f, 0.0f); }"
+          : "if (!(sig.hi > 0.0f && sig.hi < KX_INF_F)) KX_BAD_POINT");
   o("const kx_df fC = kx_df_div(cM, sig);");
   o("const kx_df lnfC = kx_df_log(fC);");
   o("const long long Tb = __double_as_longlong(T);");
@@ -1740,8 +1951,14 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
     for (int q = nw - 2; q >= 0; --q) sel = fmt("((k) < %d ? nm%d : %s)", 64 * (q + 1), q, sel.c_str());
     o("#define KX_NEG(k) ((int)((" + sel + " >> ((k) & 63)) & 1ull))");
   }
+  if (sweep) o("double Yn = Y_[i];");
   o(fmt("for (int k = 0; k < %d; ++k) {", ns));
-  o("  const double Yk = Y_[(long long)k * ld + i];");
+  if (sweep) {
+    o("  const double Yk = Yn;");
+    o(fmt("  Yn = Y_[(long long)min(k + 1, %d) * ld + i];", ns - 1));
+  } else {
+    o("  const double Yk = Y_[(long long)k * ld + i];");
+  }
   o("  const long long yb = __double_as_longlong(Yk) & 0x7fffffffffffffffLL;");
   o("  // ln |C_k| = ln |Y_k| - ln W_k + ln(C_M/sigma), floored at -700 (Y_k = 0 or |Y_k| below 1e-304: absent)");
   o("  kx_df l = kx_mk(-700.0f, 0.0f);");
@@ -1750,7 +1967,7 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
   o("    if (!(l.hi > -700.0f)) l = kx_mk(-700.0f, 0.0f);");
   o("  }");
   {
-    std::string s = "  if (Yk < 0.0) {";
+    std::string s = sweep ? "  if (__double2hiint(Yk) < 0 && yb != 0) {" : "  if (Yk < 0.0) {";
     for (int q = 0; q < nw; ++q) s += fmt(" %sif ((k >> 6) == %d) nm%d |= 1ull << (k & 63);", q ? "else " : "", q, q);
     o(s + " }");
   }
@@ -1767,7 +1984,8 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
     if (!rop) o("  w[k] = 0.0;");
   } else {
     o(lean ? "  sv[k] = make_float4(l.hi, mk_.hi, l.lo, mk_.lo);" : "  sv[k] = make_float4(l.hi, l.lo, mk_.hi, mk_.lo);");
-    if (!rop) o("  w[k] = kx_mk(0.0f, 0.0f);");
+    if (!rop && !sweep) o("  w[k] = kx_mk(0.0f, 0.0f);");
+    if (sweep) o("  KX_HU(k).x = KX_L2(l.hi, l.lo); KX_HU(k).y = KX_L2(mk_.hi, mk_.lo);");
   }
   o("}");
   {   // no negative mass fraction in this state (the usual case): the sign parities are all 0
@@ -1868,14 +2086,20 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
     o("const float lnSf = __fmul_rn(kx_i2f(S), 0.693147182f);   // S ln2 for the range tests of the scaled exponential");
   }
 
-  if (!rop && !mx && !bounded) {
+  // The class loops run over all reactions, or (listed) over those that the sweep has left; the listed form
+  // takes a fixed scale S and float pairs throughout.
+  bool listed = false;
+  std::vector<int> bit0(cls.size(), 0);   // class ci's first reaction in class order
+  for (size_t ci = 1; ci < cls.size(); ++ci) bit0[ci] = bit0[ci - 1] + (int)cls[ci - 1].rx.size();
+  auto running_scale = [&]() {
     // the state's scale 2^-S: set by its first rate (scaled to 2^62) and raised to a later rate (to
     // 2^62 again), with every accumulator rescaled, when that rate would land above 2^96.  The largest
     // scaled rate thus sits between 2^62 and 2^97, a running sum stays below ~2^116, and float pairs keep
     // their full precision for terms down to 2^-164 of the largest (anchoring the largest rate lower,
     // near 2^0, measured 5e-10 errors: rescaled partial sums fell into the subnormal range)
     o("int S = -100000;   // no rate yet");
-  }
+  };
+  if (!rop && !mx && !bounded && !sweep) running_scale();
 
   // ---- main pass, one loop per class.  Emitted twice: for warps in which some state has a
   // negative mass fraction (signed concentration products), and for the usual warps without,
@@ -1889,7 +2113,17 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
       const int E = d.nre + d.npr;
       o(fmt("{   // class %d: %d reactions, %d reactant and %d product entries", (int)ci, (int)d.rx.size(), d.nre, d.npr));
       ++o.ind;
-      prologue(d, (int)ci);
+      if (listed) {
+        o(fmt("if (lst[pos] < %d) {", bit0[ci] + (int)d.rx.size()));
+        ++o.ind;
+        o(fmt("int r = lst[pos] - %d;", bit0[ci]));
+        const int P = (E + 1 + 3) / 4 * 4;
+        o(fmt("const int4* sp4 = (const int4*)kx_s%d;", (int)ci));
+        for (int q = 0; q < P / 4; ++q) o(fmt("int4 c%d = sp4[%d * r + %d];", q, P / 4, q));
+        for (int j = 0; j < E; ++j) o(fmt("float4 v%d = sv[%s];", j, spc("c", j).c_str()));
+      } else {
+        prologue(d, (int)ci);
+      }
       if (!rop) {
         std::string pdecl = "int";
         for (int j = 0; j < E; ++j) pdecl += fmt("%s p%d = 0", j ? "," : "", j);
@@ -1897,11 +2131,20 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
         o(mx ? "double qp = 0.0;" : lean ? "float qp = 0.0f;" : "kx_df qp = kx_mk(0.0f, 0.0f);");
       }
       o("#pragma unroll 1");
-      o(fmt("for (int r = 0; r < %d; ++r) {", (int)d.rx.size()));
+      o(listed ? std::string("for (;;) {") : fmt("for (int r = 0; r < %d; ++r) {", (int)d.rx.size()));
       if (!rop)
         for (int j = 0; j < E; ++j)
           o(lean ? fmt("  const float wl%d = w[p%d & 0xffff].lo;", j, j) : fmt("  %s wl%d = w[p%d & 0xffff];", mx ? "const double" : "kx_df", j, j));
-      prefetch(d);
+      if (listed) {
+        // the next listed reaction of this class, or the record past the class's last
+        const int P = (E + 1 + 3) / 4 * 4;
+        o(fmt("  const int rn = min((int)lst[pos + 1] - %d, %d);", bit0[ci], (int)d.rx.size()));
+        for (int q = 0; q < P / 4; ++q) o(fmt("  const int4 n%d = sp4[%d * rn + %d];", q, P / 4, q));
+        for (int j = 0; j < E; ++j) o(fmt("  const float4 u%d = sv[%s];", j, spc("n", j).c_str()));
+        o(fmt("  const bool on = (kx_msk[((r + %d) >> 5) * %d + threadIdx.x] >> ((r + %d) & 31)) & 1u;", bit0[ci], opt.block, bit0[ci]));
+      } else {
+        prefetch(d);
+      }
       for (int j = 0; j < E; ++j) o(fmt("  const int k%d = %s;", j, spc("c", j).c_str()));
       if (rop) o(fmt("  const int ri = %s;", comp("c", E).c_str()));
       o(fmt("  const float4* f = kx_f%d + %d * r;", (int)ci, NF));
@@ -1955,7 +2198,7 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
         // error on the largest rates.  The estimates take the float pairs' high parts.
         // Falloff and chemically activated reactions estimate their blended ln k in float32 (the
         // same formulas as the float-pair path below, with the fast exponential and logarithm).
-        const bool fastp = !rop && opt.rates_negligible == 0 && (d.kind == Kind::Elementary || d.kind == Kind::ThreeBody || fo);
+        const bool fastp = !rop && !listed && opt.rates_negligible == 0 && (d.kind == Kind::Elementary || d.kind == Kind::ThreeBody || fo);
         if (fastp) {
           if (fo) {
             o("  const float4 f3 = f[3], f4 = f[4], f5 = f[5], f6 = f[6];");
@@ -2111,7 +2354,7 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
           c.fp32 += d.rx.size() * 4;
         } else {
           const std::string qd = fastp && !lean ? "q" : "kx_df q";
-          if (bounded) {
+          if (bounded || listed) {
             o("  " + qd + " = kx_df_mul_u(kx_df_exp_sc(L, S, lnSf), fac);   // |R| 2^-S (the products and sums after it take hi + lo as is)");
           } else {
           o("  int ex;");
@@ -2136,6 +2379,7 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
         o("  if (sf) q = kx_df_neg(q);");
         if (fastp && !lean) o("  }");
         if (d.kind == Kind::ThreeBody) { o("  q = kx_df_mul_u(q, X);"); c.fp32 += d.rx.size() * kDfMul; }
+        if (listed) o("  if (!on) q = kx_mk(0.0f, 0.0f);");
         if (lean) {
           // this rate into its accumulators at once; nothing stays pending
           for (int j = 0; j < E; ++j)
@@ -2148,7 +2392,7 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
       }
       if (rop) {
         o(mx ? "  out_[(long long)ri * ld + i] = q;" : "  out_[(long long)ri * ld + i] = kx_df2d_s(q, Sr);");
-        c.fp64 += d.rx.size();
+        (mx ? c.fp64 : c.fp32) += d.rx.size() * (mx ? 1.0 : 8.0);
       } else if (mx) {
         for (int j = 0; j < E; ++j)
           o(fmt("  { const unsigned cj = (unsigned)p%d & 0xffff0000u; if (cj != 0u) w[p%d & 0xffff] = fma(kx_f2d(__uint_as_float(cj)), qp, wl%d); }", j, j, j));
@@ -2165,6 +2409,10 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
         c.fp32 += d.rx.size() * E * (kDfAdd + kDfMulf) / 2.0;
       }
       advance(d);
+      if (listed) {
+        o("  ++pos; r = rn;");
+        o(fmt("  if (r >= %d) break;", (int)d.rx.size()));
+      }
       o("}");
       if (!rop && mx)
         for (int j = 0; j < E; ++j)
@@ -2177,27 +2425,56 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
         for (int j = 0; j < E; ++j)
           o(fmt("{ const unsigned cj = (unsigned)p%d & 0xffff0000u; if (cj != 0u) { const int kk = p%d & 0xffff; w[kk] = kx_df_add_u(w[kk], %s(qp, __uint_as_float(cj))); } }",
                 j, j, d.maxnu <= 2 ? "kx_df_scale2" : "kx_df_mulf"));
+      if (listed) { --o.ind; o("}"); }
       --o.ind;
       o("}");
     }
   };
-  o("if (__any_sync(__activemask(), anyneg)) {");
-  ++o.ind;
-  main_pass(c);
-  --o.ind;
-  o("} else {");
-  ++o.ind;
-  o("const bool anyneg = false;   // no state of this warp has a negative mass fraction");
-  {
-    OpCounts once;   // the operations are counted for one of the two copies
+  if (sweep) {
+    // every warp passes the sweep's barriers; a warp with a negative mass fraction skips its work and takes the
+    // class loops over all reactions, under a running scale
+    emit_sweep(o, g, m, cls, opt, c);
+    auto write_out = [&]() {
+      o("if (in)");
+      o("#pragma unroll 4");
+      o(fmt("for (int k = 0; k < %d; ++k) out_[(long long)k * ld + i] = bad ? KX_NAN : kx_df2d_s(w[k], S);", ns));
+    };
+    o("if (!run) {");
+    ++o.ind;
+    o(fmt("for (int k = 0; k < %d; ++k) w[k] = kx_mk(0.0f, 0.0f);", ns));
+    running_scale();
+    main_pass(c);
+    write_out();
+    --o.ind;
+    o("} else {");
+    ++o.ind;
+    o("const bool anyneg = false;");
+    OpCounts once;
+    listed = true;
     main_pass(once);
+    write_out();
+    --o.ind;
+    o("}");
+    c.fp32 += 8.0 * ns;
+  } else {
+    o("if (__any_sync(__activemask(), anyneg)) {");
+    ++o.ind;
+    main_pass(c);
+    --o.ind;
+    o("} else {");
+    ++o.ind;
+    o("const bool anyneg = false;   // no state of this warp has a negative mass fraction");
+    {
+      OpCounts once;   // the operations are counted for one of the two copies
+      main_pass(once);
+    }
+    --o.ind;
+    o("}");
   }
-  --o.ind;
-  o("}");
-  if (!rop) {
+  if (!rop && !sweep) {
     o(fmt(mx ? "for (int k = 0; k < %d; ++k) out_[(long long)k * ld + i] = w[k];"
              : "for (int k = 0; k < %d; ++k) out_[(long long)k * ld + i] = kx_df2d_s(w[k], S);", ns));
-    c.fp64 += mx ? 0 : ns;
+    c.fp32 += mx ? 0.0 : 8.0 * ns;
   }
 }
 
@@ -3731,7 +4008,7 @@ std::string emit_wdot_wc(const Mechanism& m, const EmitOptions& opt, const std::
     o("__syncwarp();");
     --o.ind;
     o("}");
-    c.fp64 += nr;
+    c.fp32 += 8.0 * nr;
     return o.o.str();
   }
   // ---- 4. the largest exponent of each state (a warp max over its rates); rates scaled in place
@@ -3792,7 +4069,7 @@ std::string emit_wdot_wc(const Mechanism& m, const EmitOptions& opt, const std::
   o("__syncwarp();");
   --o.ind;
   o("}");
-  c.fp64 += ns;
+  c.fp32 += 8.0 * ns;
   c.fp32 += ns * kDfAdd;
   return o.o.str();
 }
@@ -4492,6 +4769,9 @@ std::string emit_kernel(const Mechanism& m, KernelKind kind, const EmitOptions& 
   if (rreg == 0 && unrolled_rates) rreg = opt.mixed ? 96 : 128;
   // (large mechanisms' float-pair rates: 80, with the float32 path's short vectors; 160/900, 200003 states:
   // 3.77 ms against 4.40 at 128)
+  // the swept kernel by resident warps, not by registers: 2^20 states of 53/325 in 4.45 ms at 128 registers a
+  // thread, 3.37 at 96, 2.97 at 80, 2.57 at 64, 3.68 at 48
+  if (rreg == 0 && kind == KernelKind::Wdot && rates_swept(m, opt, false) && df_rates) rreg = 64;
   if (rreg == 0 && df_rates) rreg = opt.mixed ? 72 : (kind == KernelKind::Wdot && !opt.scratch && m.ns > 64 && opt.rates_negligible == 0) ? 80 : 128;
   if (rreg == 0 && kind == KernelKind::Transport)
     rreg = opt.tr_layout != 3 ? 128 : (!opt.mixed && opt.tr_mode == 0 && opt.part == 1 && opt.diff_mode != 2) ? 80 : 64;
@@ -4510,6 +4790,18 @@ std::string emit_kernel(const Mechanism& m, KernelKind kind, const EmitOptions& 
     for (size_t at = text.find("kx_exp("); at != std::string::npos; at = text.find("kx_exp(", at + 8)) text.replace(at, 7, "kx_exp_r(");
   }
   s << "  kx_load_tables();\n";
+  if (kind == KernelKind::Wdot && df_rates && rates_swept(m, opt, false)) {
+    // block-uniform trip count (the body holds barriers): lanes past the batch repeat its last state
+    s << "  for (long long i0 = (long long)blockIdx.x * " << opt.block << "; i0 < n; i0 += (long long)gridDim.x * " << opt.block << ") {\n"
+      << "    const bool in = i0 + threadIdx.x < n;\n"
+      << "    const long long i = in ? i0 + threadIdx.x : n - 1;\n"
+      << "    double T = T_[i], P = P_[i];\n"
+      << "    bool bad = !(T > 0.0 && P > 0.0 && T < KX_INF && P < KX_INF);\n"
+      << "    if (bad) { T = 1000.0; P = 101325.0; }\n"
+      << text << "  }\n}\n";
+    if (counts) *counts = c;
+    return s.str();
+  }
   s << "  for (long long i = (long long)blockIdx.x * " << opt.block << " + threadIdx.x; i < n; i += (long long)gridDim.x * "
     << opt.block << ") {\n";
   s << "    const double T = T_[i], P = P_[i];\n";
