@@ -83,7 +83,11 @@ typedef enum {
                     blend, ln R_f); float pairs for the Gibbs sums of ln K_c;
                     the forward-minus-reverse difference resolved from that
                     ratio and the production-rate accumulation in float64
-                    (production rates); float32 mixing rules (transport) */
+                    (production rates of more than 64 species or 400
+                    reactions; smaller mechanisms' run KX_FP64's float32 and
+                    float pairs, the faster of the two, and a state's result
+                    never depends on the states beside it); float32 mixing
+                    rules (transport) */
 } kx_precision;
 
 /* Load options; a zero-initialised struct (or NULL) selects the defaults. */
@@ -178,7 +182,7 @@ kx_status kx_mechanism_info(kx_handle h, int* n_species, int* n_reactions, doubl
  * double-float kernel evaluates a reaction in float32 when its rate is below
  * 2^-40 of its state's largest rate, where float32's error leaves the result
  * far inside the float64 bar.  Mechanisms of up to 64 species and 400
- * reactions decide this for each state by itself, unless a state of the warp
+ * reactions decide this for each state by itself (KX_MIXED always), unless a state of the warp
  * (32 consecutive states) has a negative mass fraction; larger ones, and such
  * warps, take float32 where it holds for every state of the warp: a state's
  * results can therefore differ, within the bar (~1e-11 of the per-point

@@ -433,8 +433,8 @@ kx_status kx_load_mechanism(const char* path, const kx_options* opt, kx_handle* 
       k->states_per_block = w.states_per_block;
       k->lane_use = w.lane_use;
     }
-    if (sp.kind == kx::KernelKind::Wdot && !wc_spec && k->eopt.rates_layout != 2 && (h->opt.rates_arith != 1 || k->eopt.scratch) &&
-        kx::rates_swept(h->m, k->eopt, false) && (!opt || opt->block == 0)) {
+    if (sp.kind == kx::KernelKind::Wdot && !kx::wdot_is_wc(h->m, sp.kind, k->eopt) && kx::rates_swept(h->m, k->eopt, false) &&
+        (!opt || opt->block == 0)) {
       // the warps of a block share the sweep's instruction fetches (2^20 states of 53/325 at 64 registers: blocks of
       // 128 3.59 ms, 256 2.57, 512 2.76, 1024 3.6)
       k->eopt.block = 256;

@@ -49,8 +49,9 @@
 //    than four distinct T_mid, or explicit block or register options): two
 //    float-pair Horner evaluations per species.
 //
-// The mixed-precision production rates (KX_MIXED) run the same class loops
-// with a float32 body for the Arrhenius, third-body and falloff arithmetic;
+// The mixed-precision production rates (KX_MIXED) of mechanisms without the
+// sweep (emit_sweep) and the rates of progress run the same class loops with
+// a float32 body for the Arrhenius, third-body and falloff arithmetic;
 // the Gibbs sums of ln K_c stay in float pairs (through the species
 // chemical potentials G_k/RT + ln C_k), the forward/reverse cancellation is
 // resolved from that ratio and wdot is accumulated in float64
@@ -1698,7 +1699,8 @@ std::vector<DfClass> emit_class_tables(Out& g, const Mechanism& m, bool merged =
 // pass 2 adds every reaction below 2^(M - 40) to the state's float32 sums, scaled by 2^-S, and marks the others
 // in a bit mask; the warp's marked reactions (any state's) become a list that the class loops then evaluate in
 // float pairs, each state taking those that it marked.  The choice is the state's own: its results do not
-// depend on the states beside it, but for a negative mass fraction among the warp's states (emit_rates_class_df).
+// depend on the states beside it, but for a negative mass fraction among the warp's states (emit_rates_class_df;
+// the mixed kernel's never do).
 // 2^20 states: 53/325 5.35 -> 2.57 ms, of which the species' logarithms and Gibbs energies take 25 %, pass 1
 // 18 %, pass 2 37 %, the marked reactions (16 of 325 per warp, 7 per state) 15 %, the results 18 %; 47 % of the
 // issue slots, the rest waits on the per-thread vectors (1.7 KB a state, far beyond the L1 cache).
@@ -1708,7 +1710,8 @@ void emit_sweep(Out& o, Out& g, const Mechanism& m, const std::vector<DfClass>& 
   const int W = (nr + 31) / 32;
   g("__device__ __forceinline__ float kx_ex2(float x) { float r; asm(\"ex2.approx.ftz.f32 %0, %1;\" : \"=f\"(r) : \"f\"(x)); return r; }");
   g("__device__ __forceinline__ float kx_lg2(float x) { float r; asm(\"lg2.approx.ftz.f32 %0, %1;\" : \"=f\"(r) : \"f\"(x)); return r; }");
-  o("const bool run = !__any_sync(0xffffffffu, anyneg);   // no state of this warp has a negative mass fraction");
+  // (mixed: always true, a branch around each group that keeps the compiler from merging the groups)
+  o(opt.mixed ? "const bool run = Td.hi > 0.0f;" : "const bool run = !__any_sync(0xffffffffu, anyneg);   // no state of this warp has a negative mass fraction");
   o("float tL = KX_L2(lnT.hi, lnT.lo), pL = KX_L2(lnPRT.hi, lnPRT.lo), iTf = iT.hi, Tf = Td.hi, cMf = cM.hi;");
   o("float M = -1.0e30f;");
   auto arr = [&](const Arrh& a) {   // log2 k
@@ -1816,7 +1819,8 @@ void emit_sweep(Out& o, Out& g, const Mechanism& m, const std::vector<DfClass>& 
   o("// largest scaled rate near 2^63.5; |S| < 2^11 keeps S ln2 exact to the float-pair precision");
   o("const int S = kx_rint(fminf(fmaxf(M, -1000.0f), 1000.0f)) - 63;");
   o("const float lnSf = __fmul_rn(kx_i2f(S), 0.693147182f);   // S ln2 for the range tests of the scaled exponential");
-  o("const float Sf = kx_i2f(S), thr = M - 40.0f;");
+  // (the mixed kernel's states with a negative mass fraction mark every reaction)
+  o(opt.mixed ? "const float Sf = kx_i2f(S), thr = anyneg ? -KX_INF_F : M - 40.0f;" : "const float Sf = kx_i2f(S), thr = M - 40.0f;");
   // read back, so that the second pass forms its estimates again (the compiler would keep the first pass's)
   o("volatile float back[5];");
   o("back[0] = tL; back[1] = pL; back[2] = iTf; back[3] = Tf; back[4] = cMf;");
@@ -1880,8 +1884,11 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
   // more accumulators, bound all rates first in float32 (160/900: 142-150 against 158-160 ms per 2^22
   // states with the running scale)
   const bool bounded = ns > 64;
-  // mixed precision: float32 rates, float-pair chemical potentials and Gibbs sums, float64 accumulation
-  const bool mx = opt.mixed;
+  // mixed precision: float32 rates, float-pair chemical potentials and Gibbs sums, float64 accumulation.  With
+  // the sweep the marked reactions run in float pairs for it too: 1.8e-14 of the per-point scale instead of 3e-5
+  // and no float64 sums (one multiply-add each takes 16 cycles of an SM): 53/325, 300001 states 1626 -> 779 us,
+  // 16383 312 -> 164; 9/21 118 -> 100 and 29 -> 27
+  const bool mx = opt.mixed && !rates_swept(m, opt, rop);
   std::vector<DfClass> cls = emit_class_tables(g, m);
   // With the float32 path for negligible reactions (most of them), large mechanisms' species vectors hold
   // their two high parts first, and that path touches only those and the low parts of the accumulators: 8 and
@@ -2439,22 +2446,29 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
       o("#pragma unroll 4");
       o(fmt("for (int k = 0; k < %d; ++k) out_[(long long)k * ld + i] = bad ? KX_NAN : kx_df2d_s(w[k], S);", ns));
     };
-    o("if (!run) {");
-    ++o.ind;
-    o(fmt("for (int k = 0; k < %d; ++k) w[k] = kx_mk(0.0f, 0.0f);", ns));
-    running_scale();
-    main_pass(c);
-    write_out();
-    --o.ind;
-    o("} else {");
-    ++o.ind;
-    o("const bool anyneg = false;");
-    OpCounts once;
-    listed = true;
-    main_pass(once);
-    write_out();
-    --o.ind;
-    o("}");
+    if (opt.mixed) {
+      // no second copy: a state's result never depends on the states beside it
+      listed = true;
+      main_pass(c);
+      write_out();
+    } else {
+      o("if (!run) {");
+      ++o.ind;
+      o(fmt("for (int k = 0; k < %d; ++k) w[k] = kx_mk(0.0f, 0.0f);", ns));
+      running_scale();
+      main_pass(c);
+      write_out();
+      --o.ind;
+      o("} else {");
+      ++o.ind;
+      o("const bool anyneg = false;");
+      OpCounts once;
+      listed = true;
+      main_pass(once);
+      write_out();
+      --o.ind;
+      o("}");
+    }
     c.fp32 += 8.0 * ns;
   } else {
     o("if (__any_sync(__activemask(), anyneg)) {");

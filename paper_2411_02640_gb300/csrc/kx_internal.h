@@ -85,11 +85,12 @@ struct EmitOptions {
   int rates_negligible = 0; // double-float rates: 0 float32 for reactions negligible in every state of a warp, 1 never
 };
 
-// Whether the float-pair production-rate kernel starts with the straight-line float32 sweep: its sums live in
+// Whether the production-rate kernel starts with the straight-line float32 sweep: its sums live in
 // registers, its code grows with the reactions, its marks and lists (44 bytes of marks a thread and 650 of list a
 // warp at 325 reactions) in static shared memory.
 inline bool rates_swept(const Mechanism& m, const EmitOptions& opt, bool rop) {
-  return !rop && !opt.mixed && opt.rates_negligible == 0 && m.ns <= 64 && m.nr() <= 400 && opt.block <= 512;
+  return !rop && (opt.mixed ? opt.rates_mode == 0 : opt.rates_arith != 1 || opt.scratch) && opt.rates_negligible == 0 && m.ns <= 64 &&
+         m.nr() <= 400 && opt.block <= 512;
 }
 
 // Launch shape of the warp-cooperative production-rate kernel.

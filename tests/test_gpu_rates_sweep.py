@@ -36,16 +36,17 @@ def _draw(name, n, seed):
 
 @pytest.mark.parametrize("name", ["kinds", "h2o2_9_21", "gri_53_325"])
 @pytest.mark.parametrize("n", [1, 31, 33, 255, 257, 1025])
-def test_against_float_pairs(name, n, tmp_path):
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_against_float_pairs(name, n, precision, tmp_path):
     torch = torch_cuda()
     a, b = _pair(name, tmp_path)
     T, p, Y = _draw(name, n, 40 + n)
     if n > 1:
         T[n // 2] = np.nan
     if n > 255:
-        Y[1, 40] *= -0.01     # an undershoot: its warp runs every reaction
+        Y[1, 40] *= -0.01     # an undershoot: its warp (mixed: the state itself) runs every reaction
     d = to_device(torch, T, p, Y, ld=n + 3)
-    w, r = (m.production_rates(*d)[:, :n].cpu().numpy() for m in (a, b))
+    w, r = (m.production_rates(*d, precision=q)[:, :n].cpu().numpy() for m, q in ((a, precision), (b, "fp64")))
     ok = np.isfinite(T)
     assert np.all(np.isnan(w[:, ~ok])) and np.all(np.isfinite(w[:, ok]))
     W = np.asarray(a.W)[:, None]
@@ -54,15 +55,18 @@ def test_against_float_pairs(name, n, tmp_path):
 
 
 @pytest.mark.parametrize("name", ["kinds", "gri_53_325"])
-def test_independent_of_neighbours(name, tmp_path):
-    """Without an undershoot in its warp, a state's result is the same bits wherever it stands."""
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_independent_of_neighbours(name, precision, tmp_path):
+    """Without an undershoot in its warp (mixed: whatever its warp holds), a state's result is the same bits
+    wherever it stands."""
     torch = torch_cuda()
     a, _ = _pair(name, tmp_path)
     T, p, Y = _draw(name, 700, 7)
-    w = a.production_rates(*to_device(torch, T, p, Y))
+    w = a.production_rates(*to_device(torch, T, p, Y), precision=precision)
     q = np.random.default_rng(1).permutation(700)[:413]
-    v = a.production_rates(*to_device(torch, T[q], p[q], np.ascontiguousarray(Y[:, q])))
+    v = a.production_rates(*to_device(torch, T[q], p[q], np.ascontiguousarray(Y[:, q])), precision=precision)
     assert torch.equal(v, w[:, torch.tensor(q, device="cuda")])
     Y[1, 100] = -Y[1, 100] - 1e-6
-    v = a.production_rates(*to_device(torch, T, p, Y))
-    assert torch.equal(v[:, :96], w[:, :96]) and torch.equal(v[:, 128:], w[:, 128:])
+    v = a.production_rates(*to_device(torch, T, p, Y), precision=precision)
+    lo, hi = (96, 128) if precision == "fp64" else (100, 101)
+    assert torch.equal(v[:, :lo], w[:, :lo]) and torch.equal(v[:, hi:], w[:, hi:])
