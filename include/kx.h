@@ -144,10 +144,10 @@ typedef struct {
                          only where the rate underflows); 1 one log-space exponential
                          exp(ln |R| - ln |C_k|) per entry (no reciprocal table) */
   int vjp_layout;     /* double-float adjoint: 0 (default) by batch size -- the warp-cooperative
-                         kernel for batches below min(C, 8192 w u^2) states, C the thread-per-state
+                         kernel for batches below min(C, 8192 w u^2) states (7000 above 16 species), C the thread-per-state
                          kernel's resident capacity, w the warp-cooperative kernel's resident warps
                          per SM and u the share of lane slots its class rounds fill (the crossover
-                         measured on GB300: ~8k states for 9/21, ~85k for 53/325, ~32k for
+                         measured on GB300: ~8k states for 9/21, ~95k for 53/325, ~25k for
                          160/900), one thread per state from there on; 1 always one thread per
                          state; 2 always warp-cooperative (one state per warp, its vectors and
                          per-reaction terms in shared memory, d/dC_k gathered species-major;

@@ -567,8 +567,9 @@ kx_status rop_kernel_for(kx_mech* h, int64_t n, kx_precision precision, const ch
 // state per warp) by default.  Its throughput grows with its resident warps per SM and, twice, with
 // the lane use u of its class rounds (reaction rounds and, for small mechanisms, the species
 // phases); the crossover measured on GB300 fits 8192 x resident warps per SM x u^2 states (9/21:
-// ~8k measured, 6.3k by the rule; 53/325: 65k-131k, 84k; 160/900: ~32k, 29k), and is kept below
-// the thread-per-state kernel's resident capacity.
+// ~8k measured, 6.3k by the rule) and above 16 species, whose thread-per-state kernel sums without 1/C_k, 7000 x
+// (53/325: ~77k, 95k, the two within 10 % of each other between; 160/900: 25k, 25k); it is kept below the
+// thread-per-state kernel's resident capacity.
 kx_status vjp_kernel_for(kx_mech* h, int64_t n, const char** name) {
   *name = "vjp";
   Kernel* wc = find_kernel(h, "vjp_wc");
@@ -579,7 +580,7 @@ kx_status vjp_kernel_for(kx_mech* h, int64_t n, const char** name) {
   if (s != KX_OK) return s;
   const int64_t cap = (int64_t)tps->max_blocks * tps->eopt.block;
   const double warps = (double)wc->blocks_per_sm * (wc->eopt.block / 32);
-  if (n < std::min<int64_t>(cap, (int64_t)(8192.0 * warps * wc->lane_use * wc->lane_use))) *name = "vjp_wc";
+  if (n < std::min<int64_t>(cap, (int64_t)((h->m.ns > 16 ? 7000.0 : 8192.0) * warps * wc->lane_use * wc->lane_use))) *name = "vjp_wc";
   return KX_OK;
 }
 

@@ -587,8 +587,11 @@ __device__ __forceinline__ kx_df kx_df_sub_m(kx_df m1, int e1, kx_df m2, int e2,
   const float s2 = d2 >= -126 ? __int_as_float((d2 + 127) << 23) : 0.0f;
   return kx_df_sub(kx_mk(__fmul_rn(m1.hi, s1), __fmul_rn(m1.lo, s1)), kx_mk(__fmul_rn(m2.hi, s2), __fmul_rn(m2.lo, s2)));
 }
-// A running sum as a float pair under its own scale 2^-s, 16 bytes (one load and one store).
-struct __align__(16) kx_acc { float hi, lo; int s, pad; };
+// A running sum as a float pair under its own scale 2^-s (12 bytes, or 16 in one load and store).
+#ifndef KX_ACC_ALIGN
+#define KX_ACC_ALIGN
+#endif
+struct KX_ACC_ALIGN kx_acc { float hi, lo; int s; };
 __device__ __forceinline__ void kx_acc_add(kx_df& acc, int& s, kx_df m, int e);
 __device__ __forceinline__ void kx_acc_add(kx_acc& a, kx_df m, int e) {
   kx_acc t = a;
@@ -623,6 +626,30 @@ __device__ __forceinline__ void kx_acc_add(kx_df& acc, int& s, kx_df m, int e) {
     const float sc = __int_as_float((d + 127) << 23);
     acc = kx_df_add_u(acc, kx_mk(__fmul_rn(m.hi, sc), __fmul_rn(m.lo, sc)));
   }
+}
+// The same with m in [1, 2) already (kx_acc_norm), for a term that goes to several sums.
+__device__ __forceinline__ void kx_acc_put(kx_acc& a, kx_df m, int e) {
+  if (e > a.s + 96) {
+    const int d = a.s - (e - 62);
+    const float f = d >= -126 ? __int_as_float((d + 127) << 23) : 0.0f;
+    a.hi = __fmul_rn(a.hi, f); a.lo = __fmul_rn(a.lo, f);
+    a.s = e - 62;
+  }
+  const int d = e - a.s;
+  const float sc = d >= -126 ? __int_as_float((d + 127) << 23) : 0.0f;
+  const kx_df v = kx_df_add_u(kx_mk(a.hi, a.lo), kx_mk(__fmul_rn(m.hi, sc), __fmul_rn(m.lo, sc)));
+  a.hi = v.hi; a.lo = v.lo;
+}
+// m 2^e with m brought to [1, 2); 0 far below every sum, inf and nan far above
+__device__ __forceinline__ void kx_acc_norm(kx_df& m, int& e) {
+  const float ah = fabsf(m.hi);
+  if (!(ah < KX_INF_F)) { e = 100000; m.lo = 0.0f; return; }
+  if (ah == 0.0f) { e = -200000; m.lo = 0.0f; return; }
+  const int eh = max((int)((__float_as_uint(ah) >> 23) & 0xffu) - 127, -126);
+  const int h1 = eh >> 1, h2 = eh - h1;
+  const float n1 = __int_as_float((127 - h1) << 23), n2 = __int_as_float((127 - h2) << 23);
+  m = kx_mk(__fmul_rn(__fmul_rn(m.hi, n1), n2), __fmul_rn(__fmul_rn(m.lo, n1), n2));
+  e += eh;
 }
 )KXADJ";
 
@@ -2751,8 +2778,30 @@ void emit_vjp_df(Out& o, Out& g, const Mechanism& m, OpCounts& c, bool recip) {
   o(fmt("float4 sv[%d];   // {ln |C_k| (pair), mu_k = G_k/RT + ln |C_k| (pair)}", ns));
   o(fmt("float2 yv[%d];   // Y_k/W_k (pair)", ns));
   o(fmt("float4 vh[%d];   // {cotangent v_k (pair), H_k/RT (pair)}", ns));
-  if (recip) o(fmt("float4 ic[%d];   // 1/|C_k| = {mantissa (pair), power of two (int bits), 0}", ns));
+  // Every term of a reaction's own species is R/C_k with the same C_k: gc holds their sums without it (late; the
+  // reciprocal is applied once per species at the end, the third-body terms, which lack it, are summed in gx).
+  // The kernel waits on these vectors (64 bytes per species and state, far beyond the L1 cache; 34 % of the issue
+  // slots), and a reciprocal read for each term was a fifth of what it read.  With the sums of a reaction loaded
+  // together (below) 2^18 states of 53/325: 5.49 -> 4.69 ms, 2^16 of 160/900 6.76 -> 5.72 ms.  Small mechanisms' vectors stay near and the terms take the reciprocal each (9/21,
+  // 2^18 states: 331 us, 350 the other way)
+  const bool late = recip && ns > 16;
+  if (recip && !late) o(fmt("float4 ic[%d];   // 1/|C_k| = {mantissa (pair), power of two (int bits), 0}", ns));
   o(fmt("kx_acc gc[%d];   // adjoints of C_k, each a float pair under its own scale 2^-s", ns));
+  std::vector<int> tbs;   // species with a third-body term
+  for (int k = 0; k < ns && late; ++k)
+    for (auto& r : m.rx)
+      if (r.third_body() && (r.collider >= 0 ? r.collider == k : r.eff.end() != std::find_if(r.eff.begin(), r.eff.end(), [&](const std::pair<int, double>& e) { return e.first == k; }))) {
+        tbs.push_back(k);
+        break;
+      }
+  const char* gx = late ? "gx" : "gc";
+  if (!tbs.empty()) {
+    std::string t;
+    for (int k : tbs) t += std::to_string(k) + ",";
+    g(fmt("__device__ const int kx_tbs[%d] = {%s};", (int)tbs.size(), t.c_str()));
+    o(fmt("kx_acc gx[%d];   // the third-body terms", ns));
+    o(fmt("for (int j = 0; j < %d; ++j) gx[kx_tbs[j]] = kx_acc{0.0f, 0.0f, -100000};", (int)tbs.size()));
+  }
   o("kx_df gTa = kx_mk(0.0f, 0.0f), gMa = kx_mk(0.0f, 0.0f);   // adjoints of T (fixed C) and of [M]");
   o("int sT = -100000, sM = -100000;");
   o("kx_df sig = kx_mk(0.0f, 0.0f);");
@@ -2800,8 +2849,8 @@ void emit_vjp_df(Out& o, Out& g, const Mechanism& m, OpCounts& c, bool recip) {
   o("  hk = kx_df_fma(hk, Td, KX_PF(hc + 0));");
   o("  hk = kx_df_fma(KX_PF(hc + 10), iT, hk);   // H_k/RT");
   o("  vh[k] = make_float4(vk.hi, vk.lo, hk.hi, hk.lo);");
-  if (recip) o("  { int e; const kx_df mi = kx_df_exp_m(kx_df_neg(l), e); ic[k] = make_float4(mi.hi, mi.lo, __int_as_float(e), 0.0f); }");
-  o("  gc[k] = kx_acc{0.0f, 0.0f, -100000, 0};");
+  if (recip && !late) o("  { int e; const kx_df mi = kx_df_exp_m(kx_df_neg(l), e); ic[k] = make_float4(mi.hi, mi.lo, __int_as_float(e), 0.0f); }");
+  o("  gc[k] = kx_acc{0.0f, 0.0f, -100000};");
   o("}");
   c.fp32 += 40 + 45 + kDfDiv + 3 * kDfMul + kDfAdd + kDfDiv + kDfLog;
   c.fp32 += ns * (12 + kDfFma) + ns * (45 + 2 * kDfAdd + 6 * kDfFma + kDfAdd + kDfMul);
@@ -2991,9 +3040,8 @@ void emit_vjp_df(Out& o, Out& g, const Mechanism& m, OpCounts& c, bool recip) {
       if (need_q) o("  const int eq = ef; const kx_df mq = mfs;");
       c.fp32 += NC * (2 * kDfMul + 20);
     }
-    // d/dC_k: one term per entry, R/C_k with the sign of R/C_k: as |R| = m 2^e and 1/|C_k| = m' 2^e'
-    // (per state), a product of mantissas (recip), or one log-space exponential exp(ln |R| - ln |C_k|)
-    // per entry
+    // d/dC_k: one term per entry, R/C_k with the sign of R/C_k: R = m 2^e (recip; 1/C_k at the
+    // end, or per term a product of mantissas), or one log-space exponential exp(ln |R| - ln |C_k|) per entry
     if (!recip) {
       for (int j = 0; j < E; ++j) {
         const bool reac = j < d.nre;
@@ -3002,7 +3050,7 @@ void emit_vjp_df(Out& o, Out& g, const Mechanism& m, OpCounts& c, bool recip) {
         o(fmt("    if (%s ^ KX_NEG(k%d)) mt = kx_df_neg(mt);", reac ? "sf" : "sr", j));
         o(fmt("    kx_acc_add(gc[k%d], kx_df_mul_u(%s, mt), et); }", j, reac ? aq.c_str() : ("kx_df_neg(" + aq + ")").c_str()));
       }
-    } else {
+    } else if (!late) {
       o(fmt("  { const kx_df af = kx_df_mul_u(%s, mfs);", aq.c_str()));
       if (d.rev) o(fmt("    const kx_df ar = kx_df_mul_u(%s, mr);   // mr carries the sign of R_r", ("kx_df_neg(" + aq + ")").c_str()));
       for (int j = 0; j < E; ++j) {
@@ -3013,20 +3061,41 @@ void emit_vjp_df(Out& o, Out& g, const Mechanism& m, OpCounts& c, bool recip) {
         o(fmt("      kx_acc_add(gc[k%d], mt, %s + __float_as_int(q.z)); }", j, reac ? "ef" : "er"));
       }
       o("  }");
+    } else {
+      o(fmt("  { kx_df af = kx_df_mul_u(%s, mfs);", aq.c_str()));
+      o("    int ea = ef;");
+      o("    kx_acc_norm(af, ea);");
+      if (d.rev) {
+        o(fmt("    kx_df ar = kx_df_mul_u(%s, mr);   // mr carries the sign of R_r", ("kx_df_neg(" + aq + ")").c_str()));
+        o("    int eb = er;");
+        o("    kx_acc_norm(ar, eb);");
+      }
+      const int EG = d.rev ? E : d.nre;
+      auto entry = [&](int i, int j) { return j < d.nre ? entries(m.rx[i].reac)[j] : entries(m.rx[i].prod)[j - d.nre]; };
+      // all sums of the reaction loaded before the first is stored (one at a time, each waits for the last one's
+      // store); a sum that an earlier entry of the same species has changed comes from there
+      for (int j = 0; j < EG; ++j) o(fmt("    kx_acc t%d = gc[k%d];", j, j));
+      for (int j = 0; j < EG; ++j) {
+        for (int q = 0; q < j; ++q)
+          if (std::any_of(d.rx.begin(), d.rx.end(), [&](int i) { return entry(i, j) == entry(i, q); })) o(fmt("    if (k%d == k%d) t%d = t%d;", j, q, j, q));
+        o(fmt("    kx_acc_put(t%d, %s);", j, j < d.nre ? "af, ea" : "ar, eb"));
+      }
+      for (int j = 0; j < EG; ++j) o(fmt("    gc[k%d] = t%d;", j, j));
+      o("  }");
     }
-    if (recip) c.fp32 += NC * (2 * kDfMul + E * (kDfMul + 20));
+    if (recip) c.fp32 += NC * (2 * kDfMul + E * (20 + (late ? 0 : kDfMul)));
     else c.fp32 += NC * E * (kDfAdd + kDfExp + kDfMul + 20);
     // third-body adjoint a (R_f - R_r) (times dln k_f/d[X] in a falloff), spread over [M] and the listed species
     if (tb) {
       o(d.kind == Kind::ThreeBody ? "  const kx_df gX = kx_df_mul_u(av, mq);" : "  const kx_df gX = kx_df_mul_u(kx_df_mul_u(av, mq), dX);");
       o("  if (e.y < 0) {");
       o("    const int kc = kx_effd[e.x].k;");
-      o("    kx_acc_add(gc[kc], gX, eq);");
+      o(fmt("    kx_acc_add(%s[kc], gX, eq);", gx));
       o("  } else {");
       o("    kx_acc_add(gMa, sM, kx_df_mul_u(kx_mk(f2.x, f2.y), gX), eq);");
       o("    for (int j = 0; j < e.y; ++j) {");
       o("      const kx_effd_t q = kx_effd[e.x + j];");
-      o("      kx_acc_add(gc[q.k], kx_df_mul_u(kx_mk(q.ahi, q.alo), gX), eq);");
+      o(fmt("      kx_acc_add(%s[q.k], kx_df_mul_u(kx_mk(q.ahi, q.alo), gX), eq);", gx));
       o("    }");
       o("  }");
       c.fp32 += NC * (2 * kDfMul + 4 * (kDfMul + 20));
@@ -3034,6 +3103,19 @@ void emit_vjp_df(Out& o, Out& g, const Mechanism& m, OpCounts& c, bool recip) {
     o("}");
     --o.ind;
     o("}");
+  }
+  if (late) {
+    o(fmt("for (int k = 0; k < %d; ++k) {   // the terms' common factor 1/C_k", ns));
+    o("  const float2 l = *(const float2*)&sv[k];");
+    o("  kx_acc t = gc[k];");
+    o("  int e;");
+    o("  kx_df mi = kx_df_mul_u(kx_df_norm(kx_mk(t.hi, t.lo)), kx_df_exp_m(kx_mk(-l.x, -l.y), e));");
+    o("  if (KX_NEG(k)) mi = kx_df_neg(mi);");
+    o("  t.hi = mi.hi; t.lo = mi.lo; t.s += e;");
+    o("  gc[k] = t;");
+    o("}");
+    if (!tbs.empty()) o(fmt("for (int j = 0; j < %d; ++j) { const kx_acc t = gx[kx_tbs[j]]; kx_acc_add(gc[kx_tbs[j]], kx_mk(t.hi, t.lo), t.s); }", (int)tbs.size()));
+    c.fp32 += ns * (kDfExp + kDfMul + 6) + tbs.size() * 20.0;
   }
   // ---- close the chain in float64
   o("const double iTd = 1.0 / T;");
@@ -4757,7 +4839,7 @@ std::string emit_kernel(const Mechanism& m, KernelKind kind, const EmitOptions& 
   s << "#define KX_TDF " << tdf << "\n";
   s << "#define KX_TDFR " << (df_rates || mixed_unrolled || vjp_df || kind == KernelKind::Thermo) << "\n";
   s << kTables << "\n" << kDevicePrelude << "\n";
-  if (vjp_df) s << kAdjointPrelude << "\n";
+  if (vjp_df) s << "#define KX_ACC_ALIGN " << (m.ns > 16 ? "" : "__align__(16)") << "\n" << kAdjointPrelude << "\n";
   s << "extern __shared__ __align__(16) unsigned char kx_dyn[];\n";
   s << globals.o.str();
   // the smallest index of a point outside the domain since the host last read and reset it
@@ -4790,8 +4872,10 @@ std::string emit_kernel(const Mechanism& m, KernelKind kind, const EmitOptions& 
   if (rreg == 0 && kind == KernelKind::Transport)
     rreg = opt.tr_layout != 3 ? 128 : (!opt.mixed && opt.tr_mode == 0 && opt.part == 1 && opt.diff_mode != 2) ? 80 : 64;
   if (rreg == 0 && kind == KernelKind::Thermo) rreg = 48;
-  // the double-float adjoint is bound by the latency of its local-memory vectors: residency wins
-  // (53/325, 2^18 states: 64 / 80 / 96 / 123 registers -> 6.26 / 7.16 / 7.33 / 8.58 ms)
+  // the double-float adjoint is bound by the latency of its local-memory vectors: residency wins, also where a
+  // single wave of blocks would run faster with more registers (160/900, 64 / 72 / 96 / 128 registers: 2^16 states
+  // 5.72 / 5.41 / 5.07 / 4.97 ms, 400001 21.4 / 21.0 / 25.8 / 28.4; 53/325, 64 / 72: 2^18 4.69 / 4.59, 150001
+  // 2.58 / 3.30)
   if (rreg == 0 && vjp_df) rreg = 64;
   const int min_blocks = rreg > 0 ? std::max(1, 65536 / (rreg * opt.block)) : 0;
   s << "extern \"C\" __global__ void __launch_bounds__(" << opt.block;
