@@ -541,27 +541,17 @@ template <typename V> struct kx_strided {
 // nu q for a coefficient nu in {-2, -1, 1, 2}: an exact scaling of both parts
 // (larger coefficients take the float-pair product kx_df_mulf)
 __device__ __forceinline__ kx_df kx_df_scale2(kx_df q, float nu) { return kx_mk(__fmul_rn(q.hi, nu), __fmul_rn(q.lo, nu)); }
-// (a.hi + a.lo) 2^S as a double, in integers (the float64 pipe takes 16
-// cycles of an SM per warp instruction), the power of two added to the
-// exponent field (ldexp only when the result leaves the normal range)
+// (a.hi + a.lo) 2^S as a double: one float64 addition, the power of two
+// added to the exponent field (ldexp only when the result leaves the normal
+// range)
 __device__ __forceinline__ double kx_df2d_s(kx_df a, int S) {
   if (a.hi == 0.0f && a.lo == 0.0f) return 0.0;   // (an unnormalised sum may hold its value in lo alone)
   if (!(fabsf(a.hi) < KX_INF_F)) return (double)a.hi;
-  const kx_df s = kx_ts(a.hi, a.lo);
-  const int h = __float_as_int(s.hi), e = (h >> 23) & 0xff;
-  if (e < 64 || e > 253) {
-    const double d = (double)s.hi + (double)s.lo;
-    return ldexp(d, S);
-  }
-  // hi's 24 bits as the double's leading ones, lo in units of its last (2^(e - 52); of 2^(e - 53) where hi is a
-  // power of two that lo takes the difference below), rounded once: the sum's nearest double
-  const bool dn = (h & 0x7fffff) == 0 && ((h ^ __float_as_int(s.lo)) < 0);
-  const float u = __fmul_rn(__fmul_rn(s.lo, __int_as_float((254 - e) << 23)), dn ? 0x1p53f : 0x1p52f);
-  const int l = __float2int_rn(h < 0 ? -u : u);
-  long long b = (((long long)(h & 0x7fffffff) + (896LL << 23)) << 29) + l;
-  const int E = (int)(b >> 52) + S;
-  const double d = __longlong_as_double(b | ((long long)(h & 0x80000000) << 32));
-  if (E > 0 && E < 0x7ff) return __longlong_as_double(__double_as_longlong(d) + ((long long)S << 52));
+  const double d = kx_f2d(a.hi) + kx_f2d(a.lo);
+  if (d == 0.0) return 0.0;
+  const int hi = __double2hiint(d);
+  const int E = ((hi >> 20) & 0x7ff) + S;
+  if (E > 0 && E < 0x7ff) return __hiloint2double(hi + (int)((unsigned)S << 20), __double2loint(d));
   return ldexp(d, S);
 }
 // ln(1 + y) for 0 <= y <= 1 (absolute error about 1e-15)
@@ -1735,6 +1725,28 @@ void emit_sweep(Out& o, Out& g, const Mechanism& m, const std::vector<DfClass>& 
   const int ns = m.ns, nr = m.nr();
   const double L2E = 1.4426950408889634;
   const int W = (nr + 31) / 32;
+  g(R"KXI(// (a.hi + a.lo) 2^S as a double (kx_df2d_s's value), in integers: where every thread of a full chip converts, the
+// float64 pipe's 16 cycles of an SM per warp instruction add up
+__device__ __forceinline__ double kx_df2d_i(kx_df a, int S) {
+  if (a.hi == 0.0f && a.lo == 0.0f) return 0.0;   // (an unnormalised sum may hold its value in lo alone)
+  if (!(fabsf(a.hi) < KX_INF_F)) return (double)a.hi;
+  const kx_df s = kx_ts(a.hi, a.lo);
+  const int h = __float_as_int(s.hi), e = (h >> 23) & 0xff;
+  if (e < 64 || e > 253) {
+    const double d = (double)s.hi + (double)s.lo;
+    return ldexp(d, S);
+  }
+  // hi's 24 bits as the double's leading ones, lo in units of its last (2^(e - 52); of 2^(e - 53) where hi is a
+  // power of two that lo takes the difference below), rounded once: the sum's nearest double
+  const bool dn = (h & 0x7fffff) == 0 && ((h ^ __float_as_int(s.lo)) < 0);
+  const float u = __fmul_rn(__fmul_rn(s.lo, __int_as_float((254 - e) << 23)), dn ? 0x1p53f : 0x1p52f);
+  const int l = __float2int_rn(h < 0 ? -u : u);
+  long long b = (((long long)(h & 0x7fffffff) + (896LL << 23)) << 29) + l;
+  const int E = (int)(b >> 52) + S;
+  const double d = __longlong_as_double(b | ((long long)(h & 0x80000000) << 32));
+  if (E > 0 && E < 0x7ff) return __longlong_as_double(__double_as_longlong(d) + ((long long)S << 52));
+  return ldexp(d, S);
+})KXI");
   g("__device__ __forceinline__ float kx_ex2(float x) { float r; asm(\"ex2.approx.ftz.f32 %0, %1;\" : \"=f\"(r) : \"f\"(x)); return r; }");
   g("__device__ __forceinline__ float kx_lg2(float x) { float r; asm(\"lg2.approx.ftz.f32 %0, %1;\" : \"=f\"(r) : \"f\"(x)); return r; }");
   // (mixed: always true, a branch around each group that keeps the compiler from merging the groups)
@@ -2426,7 +2438,7 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
       }
       if (rop) {
         o(mx ? "  out_[(long long)ri * ld + i] = q;" : "  out_[(long long)ri * ld + i] = kx_df2d_s(q, Sr);");
-        (mx ? c.fp64 : c.fp32) += d.rx.size() * (mx ? 1.0 : 8.0);
+        c.fp64 += d.rx.size();
       } else if (mx) {
         for (int j = 0; j < E; ++j)
           o(fmt("  { const unsigned cj = (unsigned)p%d & 0xffff0000u; if (cj != 0u) w[p%d & 0xffff] = fma(kx_f2d(__uint_as_float(cj)), qp, wl%d); }", j, j, j));
@@ -2471,7 +2483,7 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
     auto write_out = [&]() {
       o("if (in)");
       o("#pragma unroll 4");
-      o(fmt("for (int k = 0; k < %d; ++k) out_[(long long)k * ld + i] = bad ? KX_NAN : kx_df2d_s(w[k], S);", ns));
+      o(fmt("for (int k = 0; k < %d; ++k) out_[(long long)k * ld + i] = bad ? KX_NAN : kx_df2d_i(w[k], S);", ns));
     };
     if (opt.mixed) {
       // no second copy: a state's result never depends on the states beside it
@@ -2515,7 +2527,7 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
   if (!rop && !sweep) {
     o(fmt(mx ? "for (int k = 0; k < %d; ++k) out_[(long long)k * ld + i] = w[k];"
              : "for (int k = 0; k < %d; ++k) out_[(long long)k * ld + i] = kx_df2d_s(w[k], S);", ns));
-    c.fp32 += mx ? 0.0 : 8.0 * ns;
+    c.fp64 += mx ? 0 : ns;
   }
 }
 
@@ -4104,7 +4116,7 @@ std::string emit_wdot_wc(const Mechanism& m, const EmitOptions& opt, const std::
     o("__syncwarp();");
     --o.ind;
     o("}");
-    c.fp32 += 8.0 * nr;
+    c.fp64 += nr;
     return o.o.str();
   }
   // ---- 4. the largest exponent of each state (a warp max over its rates); rates scaled in place
@@ -4165,7 +4177,7 @@ std::string emit_wdot_wc(const Mechanism& m, const EmitOptions& opt, const std::
   o("__syncwarp();");
   --o.ind;
   o("}");
-  c.fp32 += 8.0 * ns;
+  c.fp64 += ns;
   c.fp32 += ns * kDfAdd;
   return o.o.str();
 }
