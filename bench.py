@@ -442,7 +442,7 @@ def run_kx(args):
             "gdof_s": value * 1e6 * (ns + 2) / 1e9,
             "mixed": {"value": world * n / (mms * 1e-3) / 1e6, "unit": "Mpoints/s", "ms_per_step": mms,
                       "kernel_ms": {k: v for k, v in zip(mnames, mper)},
-                      "dtype": "f32 + f32x2 (Gibbs sums) + f64 (wdot accumulation)",
+                      "dtype": "f32 + f32x2 (up to 64 species; larger mechanisms accumulate wdot in f64)",
                       "error": "wdot <= 2e-4 of the per-point scale max_k|W_k wdot_k| (p99 <= 1e-4); "
                                "transport <= 5e-6 relative; thermo float64-accurate",
                       "roofline": kernel_roofline(mech, mnames[mdom], n, mper[mdom], sm_max),

@@ -20,7 +20,10 @@
 //    warp vote on float32 estimates) is evaluated in float32 instead: its
 //    error, bounded by its size, stays orders of magnitude under the
 //    float-pair path's own.  The tables make the compile time independent
-//    of the mechanism's size.
+//    of the mechanism's size.  Up to 64 species and 400 reactions a
+//    straight-line float32 sweep makes that choice for each state first
+//    (emit_sweep) and the loops run over the reactions it leaves; KX_MIXED
+//    production rates are the same kernel there.
 //  * Production rates, warp-cooperative (emit_wdot_wc; small batches): the
 //    lanes of a warp share a state, species vectors and per-reaction rates
 //    in shared memory, wdot gathered species-major; the same float32 path
@@ -1721,7 +1724,7 @@ std::vector<DfClass> emit_class_tables(Out& g, const Mechanism& m, bool merged =
 // 2^20 states: 53/325 5.35 -> 2.57 ms, of which the species' logarithms and Gibbs energies take 25 %, pass 1
 // 18 %, pass 2 37 %, the marked reactions (16 of 325 per warp, 7 per state) 15 %, the results 18 %; 47 % of the
 // issue slots, the rest waits on the per-thread vectors (1.7 KB a state, far beyond the L1 cache).
-void emit_sweep(Out& o, Out& g, const Mechanism& m, const std::vector<DfClass>& cls, const EmitOptions& opt, OpCounts& c) {
+void emit_sweep(Out& o, Out& g, const Mechanism& m, const std::vector<DfClass>& cls, const EmitOptions& opt) {
   const int ns = m.ns, nr = m.nr();
   const double L2E = 1.4426950408889634;
   const int W = (nr + 31) / 32;
@@ -1912,7 +1915,6 @@ __device__ __forceinline__ double kx_df2d_i(kx_df a, int S) {
   o("if (lead) lst[cnt] = 32767;");
   o("__syncwarp();");
   o("int pos = 0;");
-  c.fp32 += nr * 50.0;
 }
 
 void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& opt, bool rop, OpCounts& c) {
@@ -2479,7 +2481,7 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
   if (sweep) {
     // every warp passes the sweep's barriers; a warp with a negative mass fraction skips its work and takes the
     // class loops over all reactions, under a running scale
-    emit_sweep(o, g, m, cls, opt, c);
+    emit_sweep(o, g, m, cls, opt);
     auto write_out = [&]() {
       o("if (in)");
       o("#pragma unroll 4");
@@ -2495,7 +2497,7 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
       ++o.ind;
       o(fmt("for (int k = 0; k < %d; ++k) w[k] = kx_mk(0.0f, 0.0f);", ns));
       running_scale();
-      main_pass(c);
+      main_pass(c);   // counted: every reaction as float-pair work, the method's work at that price
       write_out();
       --o.ind;
       o("} else {");

@@ -82,7 +82,7 @@ struct EmitOptions {
   int vjp_layout = 0;       // double-float adjoint: 0/1 thread per state, 2 warp-cooperative
   bool rop_wc = false;      // rates of progress: warp-cooperative (small batches)
   bool tr_tensor = false;   // transport sums on the tensor cores where the mechanism allows it
-  int rates_negligible = 0; // double-float rates: 0 float32 for reactions negligible in every state of a warp, 1 never
+  int rates_negligible = 0; // double-float rates: 0 float32 for negligible reactions, 1 never
 };
 
 // Whether the production-rate kernel starts with the straight-line float32 sweep: its sums live in
