@@ -1753,7 +1753,7 @@ __device__ __forceinline__ double kx_df2d_i(kx_df a, int S) {
   g("__device__ __forceinline__ float kx_ex2(float x) { float r; asm(\"ex2.approx.ftz.f32 %0, %1;\" : \"=f\"(r) : \"f\"(x)); return r; }");
   g("__device__ __forceinline__ float kx_lg2(float x) { float r; asm(\"lg2.approx.ftz.f32 %0, %1;\" : \"=f\"(r) : \"f\"(x)); return r; }");
   // (mixed: always true, a branch around each group that keeps the compiler from merging the groups)
-  o(opt.mixed ? "const bool run = Td.hi > 0.0f;" : "const bool run = !__any_sync(0xffffffffu, anyneg);   // no state of this warp has a negative mass fraction");
+  o(opt.mixed ? "const bool run = Td.hi > 0.0f;" : "const bool run = !__any_sync(0xffffffffu, anyneg && !bad);   // no state of this warp has a negative mass fraction");
   o("float tL = KX_L2(lnT.hi, lnT.lo), pL = KX_L2(lnPRT.hi, lnPRT.lo), iTf = iT.hi, Tf = Td.hi, cMf = cM.hi;");
   o("float M = -1.0e30f;");
   auto arr = [&](const Arrh& a) {   // log2 k
@@ -1910,7 +1910,7 @@ __device__ __forceinline__ double kx_df2d_i(kx_df a, int S) {
   o("int cnt = 0;");
   o("__syncwarp();");
   for (int w = 0; w < W; ++w) {
-    o(fmt("for (unsigned a = __reduce_or_sync(0xffffffffu, run ? kx_msk[%d + threadIdx.x] : 0u); a; a &= a - 1) { if (lead) lst[cnt] = (short)(%d + __ffs(a) - 1); ++cnt; }", w * opt.block, 32 * w));
+    o(fmt("for (unsigned a = __reduce_or_sync(0xffffffffu, run && !bad ? kx_msk[%d + threadIdx.x] : 0u); a; a &= a - 1) { if (lead) lst[cnt] = (short)(%d + __ffs(a) - 1); ++cnt; }", w * opt.block, 32 * w));
   }
   o("if (lead) lst[cnt] = 32767;");
   o("__syncwarp();");
@@ -2482,6 +2482,7 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
     // every warp passes the sweep's barriers; a warp with a negative mass fraction skips its work and takes the
     // class loops over all reactions, under a running scale
     emit_sweep(o, g, m, cls, opt);
+    o("if (in && bad) atomicMin(&kx_bad_first, (unsigned long long)i);   // a point outside the domain");
     auto write_out = [&]() {
       o("if (in)");
       o("#pragma unroll 4");
