@@ -1586,6 +1586,21 @@ void emit_class_mixed_body(Out& o, const DfClass& d, int ci, int E, OpCounts& c)
   }
 }
 
+// Net efficiency of every species; and whether [X] = e_default C_M + sum (e_k - e_default) C_k may cancel: float32
+// gives it to 2^-20 or so while no efficiency is below a quarter of the default ([X] >= e_default C_M/4), and to
+// noise of 2^-22 C_M, of either sign, in a mixture of species with efficiency 0.
+std::vector<double> net_eff(const Reaction& r, int ns) {
+  std::vector<double> e(ns, r.default_eff);
+  for (auto& x : r.eff) e[x.first] += x.second - r.default_eff;
+  return e;
+}
+bool third_body_cancels(const Reaction& r, int ns) {
+  if (!r.third_body() || r.collider >= 0) return false;
+  for (double e : net_eff(r, ns))
+    if (e < 0.25 * r.default_eff) return true;
+  return false;
+}
+
 // Reaction classes of one code shape and their constant tables: per class the
 // packed species entries (kx_s<c>), the Arrhenius / blend records (kx_f<c>) and
 // the efficiency / PLOG index pairs (kx_e<c>); the efficiencies, PLOG tables
@@ -1769,6 +1784,14 @@ __device__ __forceinline__ double kx_df2d_i(kx_df a, int S) {
       std::string X;
       if (r.collider >= 0) {
         X = fmt("kx_ex2(h%d)", r.collider);
+      } else if (third_body_cancels(r, ns)) {
+        // all species' own terms, none of them negative
+        const std::vector<double> eff = net_eff(r, ns);
+        X = "0.0f";
+        for (int k = 0; k < ns; ++k) {
+          if (eff[k] < 0.0 && !bound) return std::string();   // (a species listed twice) always marked
+          if (eff[k] != 0.0) X = fmt("fmaf(%s, kx_ex2(((const volatile float2&)KX_HU(%d)).x), %s)", F(std::fabs(eff[k])).c_str(), k, X.c_str());
+        }
       } else {
         X = fmt("%s * cMf", F(r.default_eff).c_str());
         for (auto& x : r.eff)
@@ -1795,7 +1818,7 @@ __device__ __forceinline__ double kx_df2d_i(kx_df a, int S) {
       t += "const float l1 = kx_lg2(1.0f + kx_ex2(-fabsf(lp))); ";
       t += r.kind == Kind::Falloff ? "float e = ki + (lp < 0.0f ? lp - l1 : -l1) + lF; " : "float e = k0 + lF - (lp < 0.0f ? l1 : lp + l1); ";
     } else if (r.kind == Kind::Plog) {
-      if (!bound) return std::string();   // always marked
+      if (!bound) return std::string();
       t += "float e, k1; e = k1 = " + arr(Arrh{r.plog[0][1], r.plog[0][2], r.plog[0][3]}) + "; ";
       for (size_t j = 1; j < r.plog.size(); ++j) {   // between pressures j - 1 and j, or above j
         const double l0 = std::log(r.plog[j - 1][0]), l1 = std::log(r.plog[j][0]);
@@ -1839,7 +1862,8 @@ __device__ __forceinline__ double kx_df2d_i(kx_df a, int S) {
       const Reaction& r = m.rx[order[q]];
       for (auto& e : r.reac) need[e.first] |= r.reversible ? 3 : 1;
       for (auto& e : r.prod) need[e.first] |= r.reversible ? 2 : 0;
-      for (auto& e : r.eff) need[e.first] |= 1;
+      if (!third_body_cancels(r, ns))
+        for (auto& e : r.eff) need[e.first] |= 1;
       if (r.collider >= 0) need[r.collider] |= 1;
     }
     for (int k = 0; k < ns; ++k) {
@@ -1884,8 +1908,9 @@ __device__ __forceinline__ double kx_df2d_i(kx_df a, int S) {
       const std::string mark = fmt("mw |= 0x%xu;", 1u << (bit % 32));
       ++bit;
       const std::string put = bit % 32 && bit != nr ? std::string() : fmt(" kx_msk[%d + threadIdx.x] = mw; mw = 0u;", (bit - 1) / 32 * opt.block);
-      if (r.kind == Kind::Plog) { o(mark + put); continue; }
-      std::string t = "{ " + estimate(r, false);
+      const std::string est = estimate(r, false);
+      if (est.empty()) { o(mark + put); continue; }   // always in float pairs
+      std::string t = "{ " + est;
       t += "const bool p = " + largest(r) + " < thr; if (!p) " + mark + " ";
       t += r.reversible ? "float q = kx_ex2(e - Sf) - kx_ex2(r - Sf); " : "float q = kx_ex2(e - Sf); ";
       t += "q = p ? q : 0.0f;";
@@ -1938,6 +1963,9 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
   // 3.75 at 80 registers.  53/325 gained nothing from it (traffic from L2 halved, 18 % fewer instructions, the
   // float-pair path's own loads no longer ahead of time: 5.41 -> 5.60 ms) and keeps the full loads.
   const bool lean = !rop && !mx && opt.rates_negligible == 0 && bounded;
+  auto cancels = [&](const DfClass& d) {
+    return std::any_of(d.rx.begin(), d.rx.end(), [&](int i) { return third_body_cancels(m.rx[i], ns); });
+  };
   // Small mechanisms: a straight-line float32 sweep over all reactions first (emit_sweep), the class loops for
   // those that it leaves
   const bool sweep = rates_swept(m, opt, rop);
@@ -2077,6 +2105,21 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
 
   if (mx) o("const float lnTf = lnT.hi, iTf = iT.hi, Tf = Td.hi, cMf = cM.hi;");
   if (mx && any_plog) o("const float lnPf = lnP.hi;");
+  auto third_body_f32 = [&]() {
+    o("  float Xf = 0.0f;");
+    o("  if (e.y < 0) {");
+    o("    const int kc = kx_effd[e.x].k;");
+    o("    Xf = __expf(KX_SVH(kc).x);");
+    o("    if (anyneg && KX_NEG(kc)) Xf = -Xf;");
+    o("  } else {");
+    o("    for (int j = 0; j < e.y; ++j) {");
+    o("      const kx_effd_t q = kx_effd[e.x + j];");
+    o("      const float C = __expf(KX_SVH(q.k).x);");
+    o("      Xf = fmaf(q.ahi, anyneg && KX_NEG(q.k) ? -C : C, Xf);");
+    o("    }");
+    o("    Xf = fmaf(f2.x, cM.hi, Xf);");
+    o("  }");
+  };
   if (!rop && !mx && bounded) {
     o("const float lnTf = lnT.hi, iTf = iT.hi, Tf = Td.hi, lnPRTf = lnPRT.hi, lncMf = __logf(cM.hi);");
     o("float U = -1.0e30f;");
@@ -2096,7 +2139,15 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
       o(d.kconst ? "  float b = f0.x;" : "  float b = fmaf(f0.z, lnTf, fmaf(f1.x, iTf, f0.x));");
       if (d.kind == Kind::ThreeBody) {
         o(fmt("  const int2 e = kx_e%d[r];", (int)ci));
-        o("  b += e.y < 0 ? sv[kx_effd[e.x].k].x : lncMf + f1.z;");
+        if (lean && cancels(d)) {
+          // (the largest efficiency's bound would be far above the rate in a mixture of species with efficiency
+          // 0, and with it what counts as negligible)
+          o("  const float4 f2 = f[2];");
+          third_body_f32();
+          o("  b += e.y < 0 ? sv[kx_effd[e.x].k].x : __logf(fmaf(0x1p-20f * f2.x, cM.hi, fabsf(Xf)));");
+        } else {
+          o("  b += e.y < 0 ? sv[kx_effd[e.x].k].x : lncMf + f1.z;");
+        }
       } else if (fo) {
         o("  const float4 f2 = f[2], f3 = f[3], f4 = f[4], f5 = f[5], f6 = f[6];");
         o("  // ln F <= max(0, ln F_cent) (Troe); ln d + e ln T + max(0, ln base) (SRI)");
@@ -2106,7 +2157,13 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
           o("  const float lf = f5.z + f6.x * lnTf + fmaxf(0.0f, __logf(f4.x * __expf(f4.z * iTf) + __expf(Tf * f5.x)));");
         else
           o("  const float lf = 0.0f;");
-        if (d.kind == Kind::ChemAct) o("  b = fmaf(f3.x, lnTf, fmaf(f3.z, iTf, f2.z)) + lf;");
+        if (lean && d.kind == Kind::Falloff && cancels(d)) {
+          // k_inf F Pr/(1 + Pr) <= min(k_inf, k_0 [X]) F
+          o(fmt("  const int2 e = kx_e%d[r];", (int)ci));
+          third_body_f32();
+          o("  const float lX = e.y < 0 ? sv[kx_effd[e.x].k].x : __logf(fmaf(0x1p-20f * f2.x, cM.hi, fabsf(Xf)));");
+          o("  b = fminf(b, fmaf(f3.x, lnTf, fmaf(f3.z, iTf, f2.z)) + lX) + lf;");
+        } else if (d.kind == Kind::ChemAct) o("  b = fmaf(f3.x, lnTf, fmaf(f3.z, iTf, f2.z)) + lf;");
         else o("  b += lf;");
       } else if (d.kind == Kind::Plog) {
         o(fmt("  const int2 e = kx_e%d[r];", (int)ci));
@@ -2221,19 +2278,9 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
           if (lean) {
             // [X] in float32 from C = e^ln|C| (off by the logarithm's 4e-5, as the rates of this path are);
             // the float-pair path forms its own
-            o("  float Xf = 0.0f;");
-            o("  if (e.y < 0) {");
-            o("    const int kc = kx_effd[e.x].k;");
-            o("    Xf = __expf(KX_SVH(kc).x);");
-            o("    if (anyneg && KX_NEG(kc)) Xf = -Xf;");
-            o("  } else {");
-            o("    for (int j = 0; j < e.y; ++j) {");
-            o("      const kx_effd_t q = kx_effd[e.x + j];");
-            o("      const float C = __expf(KX_SVH(q.k).x);");
-            o("      Xf = fmaf(q.ahi, anyneg && KX_NEG(q.k) ? -C : C, Xf);");
-            o("    }");
-            o("    Xf = fmaf(f2.x, cM.hi, Xf);");
-            o("  }");
+            third_body_f32();
+            // (cancelled to noise, of a quantity that may be the largest rate's: no float32 path)
+            if (cancels(d)) o("  if (e.y >= 0 && !(Xf >= 0x1p-10f * f2.x * cM.hi)) Xf = __int_as_float(0x7fffffff);");
           } else {
             third_body_df();
           }
