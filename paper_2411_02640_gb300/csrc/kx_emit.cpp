@@ -2856,7 +2856,7 @@ void emit_vjp_df(Out& o, Out& g, const Mechanism& m, OpCounts& c, bool recip) {
         tbs.push_back(k);
         break;
       }
-  const char* gx = late ? "gx" : "gc";
+  const char* gx = late && !tbs.empty() ? "gx" : "gc";   // (no such species: the third-body loops are empty)
   if (!tbs.empty()) {
     std::string t;
     for (int k : tbs) t += std::to_string(k) + ",";
