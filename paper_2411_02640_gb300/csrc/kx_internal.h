@@ -87,9 +87,9 @@ struct EmitOptions {
 
 // Whether the production-rate kernel starts with the straight-line float32 sweep: its sums live in
 // registers, its code grows with the reactions, its marks and lists (44 bytes of marks a thread and 650 of list a
-// warp at 325 reactions) in static shared memory.
+// warp at 325 reactions) in static shared memory.  (Without reactions there is nothing to sweep.)
 inline bool rates_swept(const Mechanism& m, const EmitOptions& opt, bool rop) {
-  return !rop && (opt.mixed ? opt.rates_mode == 0 : opt.rates_arith != 1 || opt.scratch) && opt.rates_negligible == 0 && m.ns <= 64 &&
+  return !rop && m.nr() > 0 && (opt.mixed ? opt.rates_mode == 0 : opt.rates_arith != 1 || opt.scratch) && opt.rates_negligible == 0 && m.ns <= 64 &&
          m.nr() <= 400 && opt.block <= 512;
 }
 
