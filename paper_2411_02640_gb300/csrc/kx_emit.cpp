@@ -2443,13 +2443,21 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
           o("  }");
           c.fp32 += d.rx.size() * ((E - 1) * kDfAdd + (dn ? kDfAdd + kDfMulf : 0) + kDfAdd + kDfExp + 10);
         }
+        const bool xscaled = d.kind == Kind::ThreeBody && !rop && (bounded || listed);
         if (rop) {
           o("  const int Sr = kx_rint(fminf(fmaxf(L.hi * KX_LOG2E_F, -1000.0f), 1000.0f));");
           o("  kx_df q = kx_df_mul_u(kx_df_exp_sc(L, Sr, __fmul_rn(kx_i2f(Sr), 0.693147182f)), fac);");
           c.fp32 += d.rx.size() * 4;
         } else {
           const std::string qd = fastp && !lean ? "q" : "kx_df q";
-          if (bounded || listed) {
+          if (xscaled) {
+            // [X] multiplies last; its power of two goes into the scale before, which bounds the rate with [X]
+            // (without it the rate of a trace collider lies any distance above)
+            o("  const int ex = min(max((int)((__float_as_uint(X.hi) >> 23) & 0xffu) - 127, -126), 126);");
+            o("  const float xs = __int_as_float((127 - ex) << 23);");
+            o("  const kx_df Xs = kx_mk(__fmul_rn(X.hi, xs), __fmul_rn(X.lo, xs));");
+            o("  " + qd + " = kx_df_mul_u(kx_df_exp_sc(L, S - ex, __fmul_rn(kx_i2f(S - ex), 0.693147182f)), fac);   // |R|/[X] 2^(ex - S)");
+          } else if (bounded || listed) {
             o("  " + qd + " = kx_df_mul_u(kx_df_exp_sc(L, S, lnSf), fac);   // |R| 2^-S (the products and sums after it take hi + lo as is)");
           } else {
           o("  int ex;");
@@ -2473,7 +2481,7 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
         }
         o("  if (sf) q = kx_df_neg(q);");
         if (fastp && !lean) o("  }");
-        if (d.kind == Kind::ThreeBody) { o("  q = kx_df_mul_u(q, X);"); c.fp32 += d.rx.size() * kDfMul; }
+        if (d.kind == Kind::ThreeBody) { o(xscaled ? "  q = kx_df_mul_u(q, Xs);" : "  q = kx_df_mul_u(q, X);"); c.fp32 += d.rx.size() * kDfMul; }
         if (listed) o("  if (!on) q = kx_mk(0.0f, 0.0f);");
         if (lean) {
           // this rate into its accumulators at once; nothing stays pending
