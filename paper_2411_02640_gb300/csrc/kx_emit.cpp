@@ -4168,7 +4168,8 @@ std::string emit_wdot_wc(const Mechanism& m, const EmitOptions& opt, const std::
     o("  const int flag = sci[g].y;");
     o("  if (flag == 2) continue;");
     o(fmt("  const float2 q = qm[%d * g + r];", nr));
-    o(fmt("  out_[(long long)r * ld + i0 + g] = flag == 1 ? KX_NAN : kx_df2d_s(kx_df_norm(kx_mk(q.x, q.y)), (int)qe[%d * g + r]);", nr));
+    o("  const kx_df m = fabsf(q.x) < KX_INF_F ? kx_df_norm(kx_mk(q.x, q.y)) : kx_mk(q.x, 0.0f);   // (beyond float64: inf, its low part nan)");
+    o(fmt("  out_[(long long)r * ld + i0 + g] = flag == 1 ? KX_NAN : kx_df2d_s(m, (int)qe[%d * g + r]);", nr));
     o("}");
     o(fmt("if (lane < %d && sci[lane].y == 1) atomicMin(&kx_bad_first, (unsigned long long)(i0 + lane));", G));
     o("__syncwarp();");
