@@ -182,8 +182,9 @@ kx_status kx_mechanism_info(kx_handle h, int* n_species, int* n_reactions, doubl
  * double-float kernel evaluates a reaction in float32 when its rate is below
  * 2^-40 of its state's largest rate, where float32's error leaves the result
  * far inside the float64 bar.  Mechanisms of up to 64 species and 400
- * reactions decide this for each state by itself (KX_MIXED always), unless a state of the warp
- * (32 consecutive states) has a negative mass fraction; larger ones, and such
+ * reactions decide this for each state by itself, undershoots included
+ * (KX_MIXED always; KX_FP64 unless the negative mass fractions of a state of the warp, 32
+ * consecutive states, make up more than 2^-6 of its sum Y/W); larger mechanisms, and such
  * warps, take float32 where it holds for every state of the warp: a state's
  * results can therefore differ, within the bar (~1e-11 of the per-point
  * scale), with the states it shares a warp with (a call on a sub-range that

@@ -1734,8 +1734,10 @@ std::vector<DfClass> emit_class_tables(Out& g, const Mechanism& m, bool merged =
 // pass 2 adds every reaction below 2^(M - 40) to the state's float32 sums, scaled by 2^-S, and marks the others
 // in a bit mask; the warp's marked reactions (any state's) become a list that the class loops then evaluate in
 // float pairs, each state taking those that it marked.  The choice is the state's own: its results do not
-// depend on the states beside it, but for a negative mass fraction among the warp's states (emit_rates_class_df;
-// the mixed kernel's never do).
+// depend on the states beside it, but (KX_FP64) for large negative mass fractions among the warp's states.
+// Warps with negative mass fractions take pass 2 with the signs of the concentration products (a copy of its own:
+// one copy with signs for all cost the others 6 %).  2^18 states of 53/325, 1 % of the mass fractions negative:
+// 0.83 ms, 0.72 without, against 2.24 (mixed 2.53) with every reaction in the class loops.
 // 2^20 states: 53/325 5.35 -> 2.57 ms, of which the species' logarithms and Gibbs energies take 25 %, pass 1
 // 18 %, pass 2 37 %, the marked reactions (16 of 325 per warp, 7 per state) 15 %, the results 18 %; 47 % of the
 // issue slots, the rest waits on the per-thread vectors (1.7 KB a state, far beyond the L1 cache).
@@ -1767,8 +1769,13 @@ __device__ __forceinline__ double kx_df2d_i(kx_df a, int S) {
 })KXI");
   g("__device__ __forceinline__ float kx_ex2(float x) { float r; asm(\"ex2.approx.ftz.f32 %0, %1;\" : \"=f\"(r) : \"f\"(x)); return r; }");
   g("__device__ __forceinline__ float kx_lg2(float x) { float r; asm(\"lg2.approx.ftz.f32 %0, %1;\" : \"=f\"(r) : \"f\"(x)); return r; }");
-  // (mixed: always true, a branch around each group that keeps the compiler from merging the groups)
-  o(opt.mixed ? "const bool run = Td.hi > 0.0f;" : "const bool run = !__any_sync(0xffffffffu, anyneg && !bad);   // no state of this warp has a negative mass fraction");
+  // Undershoots take the sweep with signs.  Where the negative species make up more than 2^-6 of sum |Y/W|, its bounds
+  // do not hold: such a state marks every reaction (mixed), or its warp takes the class loops over all reactions.
+  o("const bool heavy = !bad && sneg > 0x1p-6f * sig.hi;");
+  o("const bool sgn = __any_sync(0xffffffffu, anyneg && !bad);   // some state of this warp has a negative mass fraction");
+  o("const unsigned nlo = (unsigned)nm0, nhi = (unsigned)(nm0 >> 32);");
+  o("const bool once = __any_sync(0xffffffffu, Td.hi > 0.0f);   // always true: a branch around each group that keeps the compiler from merging them");
+  o(opt.mixed ? "const bool run = once;" : "const bool run = !__any_sync(0xffffffffu, heavy);");
   o("float tL = KX_L2(lnT.hi, lnT.lo), pL = KX_L2(lnPRT.hi, lnPRT.lo), iTf = iT.hi, Tf = Td.hi, cMf = cM.hi;");
   o("float M = -1.0e30f;");
   auto arr = [&](const Arrh& a) {   // log2 k
@@ -1778,26 +1785,44 @@ __device__ __forceinline__ double kx_df2d_i(kx_df a, int S) {
     return t;
   };
   // float e = log2 |R_f|, r = log2 |R_r|
-  auto estimate = [&](const Reaction& r, bool bound) {
+  // (sgn: of states with negative mass fractions, whose species' signs are the bits of nlo, nhi)
+  auto neg = [&](int k) { return k < 32 ? fmt("(nlo >> %d)", k) : fmt("(nhi >> %d)", k - 32); };
+  auto estimate = [&](const Reaction& r, bool bound, bool sgn = false) {
+    auto conc = [&](const std::string& h, int k) {   // C_k from its logarithm
+      return sgn ? fmt("__uint_as_float(__float_as_uint(kx_ex2(%s)) ^ (%s << 31))", h.c_str(), neg(k).c_str()) : "kx_ex2(" + h + ")";
+    };
+    auto hu = [](int k) { return fmt("((const volatile float2&)KX_HU(%d)).x", k); };
     std::string t;
     if (r.third_body()) {
-      std::string X;
+      std::string X, A;   // [X], and the sum of its terms' magnitudes
+      bool below = false;
       if (r.collider >= 0) {
-        X = fmt("kx_ex2(h%d)", r.collider);
+        X = conc(fmt("h%d", r.collider), r.collider);
       } else if (third_body_cancels(r, ns)) {
         // all species' own terms, none of them negative
         const std::vector<double> eff = net_eff(r, ns);
-        X = "0.0f";
+        X = A = "0.0f";
         for (int k = 0; k < ns; ++k) {
           if (eff[k] < 0.0 && !bound) return std::string();   // (a species listed twice) always marked
-          if (eff[k] != 0.0) X = fmt("fmaf(%s, kx_ex2(((const volatile float2&)KX_HU(%d)).x), %s)", F(std::fabs(eff[k])).c_str(), k, X.c_str());
+          if (eff[k] == 0.0) continue;
+          X = fmt("fmaf(%s, %s, %s)", F(std::fabs(eff[k])).c_str(), conc(hu(k), k).c_str(), X.c_str());
+          A = fmt("fmaf(%s, kx_ex2(%s), %s)", F(std::fabs(eff[k])).c_str(), hu(k).c_str(), A.c_str());
         }
       } else {
-        X = fmt("%s * cMf", F(r.default_eff).c_str());
-        for (auto& x : r.eff)
-          if (x.second != r.default_eff) X = fmt("fmaf(%s, kx_ex2(h%d), %s)", F(x.second - r.default_eff).c_str(), x.first, X.c_str());
+        X = A = fmt("%s * cMf", F(r.default_eff).c_str());
+        for (auto& x : r.eff) {
+          const double de = x.second - r.default_eff;
+          if (de == 0.0) continue;
+          below |= de < 0.0;
+          X = fmt("fmaf(%s, %s, %s)", F(de).c_str(), conc(fmt("h%d", x.first), x.first).c_str(), X.c_str());
+          A = fmt("fmaf(%s, kx_ex2(h%d), %s)", F(std::fabs(de)).c_str(), x.first, A.c_str());
+        }
       }
-      t += "const float X = " + X + ", x = kx_lg2(X); ";
+      t += "float X = " + X + "; ";
+      if (sgn && r.collider < 0) t += "X = X >= 0x1p-10f * (" + A + ") ? X : __int_as_float(0x7fffffff); ";   // (cancelled: marked)
+      // (the terms' magnitudes are summed here: only a large negative mass fraction leaves less than that)
+      if (bound && opt.mixed && below) t += fmt("X = fmaxf(fabsf(X), %s * cMf); ", F(std::ldexp(r.default_eff, -20)).c_str());
+      t += sgn && r.kind == Kind::ThreeBody ? "const float x = kx_lg2(fabsf(X)); " : "const float x = kx_lg2(X); ";
     }
     if (r.kind == Kind::Falloff || r.kind == Kind::ChemAct) {
       t += "const float ki = " + arr(r.k) + ", k0 = " + arr(r.k0) + ", lp = k0 - ki + x; ";
@@ -1885,50 +1910,67 @@ __device__ __forceinline__ double kx_df2d_i(kx_df a, int S) {
   o("// largest scaled rate near 2^63.5; |S| < 2^11 keeps S ln2 exact to the float-pair precision");
   o("const int S = kx_rint(fminf(fmaxf(M, -1000.0f), 1000.0f)) - 63;");
   o("const float lnSf = __fmul_rn(kx_i2f(S), 0.693147182f);   // S ln2 for the range tests of the scaled exponential");
-  // (the mixed kernel's states with a negative mass fraction mark every reaction)
-  o(opt.mixed ? "const float Sf = kx_i2f(S), thr = anyneg ? -KX_INF_F : M - 40.0f;" : "const float Sf = kx_i2f(S), thr = M - 40.0f;");
+  o(opt.mixed ? "const float Sf = kx_i2f(S), thr = heavy ? -KX_INF_F : M - 40.0f;" : "const float Sf = kx_i2f(S), thr = M - 40.0f;");
   // read back, so that the second pass forms its estimates again (the compiler would keep the first pass's)
   o("volatile float back[5];");
   o("back[0] = tL; back[1] = pL; back[2] = iTf; back[3] = Tf; back[4] = cMf;");
   o("tL = back[0]; pL = back[1]; iTf = back[2]; Tf = back[3]; cMf = back[4];");
+  std::string sums;
   {
     std::string a;
     for (int k = 0; k < ns; ++k) a += fmt("%sa%d = 0.0f", k ? ", " : "float ", k);
-    o(a + ";");
+    sums = a + ";";
     o(fmt("__shared__ unsigned kx_msk[%d];", W * opt.block));
     o("unsigned mw = 0u;   // marks of 32 reactions");
   }
-  o("// pass 2: negligible reactions into the float32 sums, the others marked");
-  int bit = 0;
-  at = 0;
-  for (auto& d : cls)
-    for (int i : d.rx) {
-      group();
-      const Reaction& r = m.rx[i];
-      const std::string mark = fmt("mw |= 0x%xu;", 1u << (bit % 32));
-      ++bit;
-      const std::string put = bit % 32 && bit != nr ? std::string() : fmt(" kx_msk[%d + threadIdx.x] = mw; mw = 0u;", (bit - 1) / 32 * opt.block);
-      const std::string est = estimate(r, false);
-      if (est.empty()) { o(mark + put); continue; }   // always in float pairs
-      std::string t = "{ " + est;
-      t += "const bool p = " + largest(r) + " < thr; if (!p) " + mark + " ";
-      t += r.reversible ? "float q = kx_ex2(e - Sf) - kx_ex2(r - Sf); " : "float q = kx_ex2(e - Sf); ";
-      t += "q = p ? q : 0.0f;";
-      std::map<int, int> net;
-      for (auto& e : r.reac) net[e.first] -= e.second;
-      for (auto& e : r.prod) net[e.first] += e.second;
-      for (auto& kv : net) {
-        if (kv.second == 1) t += fmt(" a%d += q;", kv.first);
-        else if (kv.second == -1) t += fmt(" a%d -= q;", kv.first);
-        else if (kv.second != 0) t += fmt(" a%d = fmaf(%s, q, a%d);", kv.first, F(kv.second).c_str(), kv.first);
-      }
-      o(t + " }" + put);
+  o("// pass 2: negligible reactions into the float32 sums, the others marked; with signs where the warp has negative mass fractions");
+  auto second = [&](int q, bool sgn) {
+    const Reaction& r = m.rx[order[q]];
+    const std::string mark = fmt("mw |= 0x%xu;", 1u << (q % 32));
+    const std::string put = (q + 1) % 32 && q + 1 != nr ? std::string() : fmt(" kx_msk[%d + threadIdx.x] = mw; mw = 0u;", q / 32 * opt.block);
+    const std::string est = estimate(r, false, sgn);
+    if (est.empty()) { o(mark + put); return; }   // always in float pairs
+    auto rate = [&](const char* e, const std::vector<int>& side) {
+      const std::string v = fmt("kx_ex2(%s - Sf)", e);
+      std::string x = r.kind == Kind::ThreeBody ? "(__float_as_uint(X) >> 31)" : "";
+      for (int k : side) x += (x.empty() ? "" : " ^ ") + neg(k);
+      return sgn && !x.empty() ? "__uint_as_float(__float_as_uint(" + v + ") ^ ((" + x + ") << 31))" : v;
+    };
+    std::string t = "{ " + est;
+    t += "const bool p = " + largest(r) + " < thr; if (!p) " + mark + " ";
+    t += "float q = " + rate("e", entries(r.reac)) + (r.reversible ? " - " + rate("r", entries(r.prod)) : "") + "; ";
+    t += "q = p ? q : 0.0f;";
+    std::map<int, int> net;
+    for (auto& e : r.reac) net[e.first] -= e.second;
+    for (auto& e : r.prod) net[e.first] += e.second;
+    for (auto& kv : net) {
+      if (kv.second == 1) t += fmt(" a%d += q;", kv.first);
+      else if (kv.second == -1) t += fmt(" a%d -= q;", kv.first);
+      else if (kv.second != 0) t += fmt(" a%d = fmaf(%s, q, a%d);", kv.first, F(kv.second).c_str(), kv.first);
     }
-  o("}");
-  o("// the sums start the float-pair accumulators; the warp's list of marked reactions, in class order");
-  o("if (run) {");
-  for (int k = 0; k < ns; ++k) o(fmt("w[%d] = kx_mk(a%d, 0.0f);", k, k));
-  o("}");
+    o(t + " }" + put);
+  };
+  // A copy for each kind of warp, its sums in registers throughout; every warp passes as many barriers.  (With the
+  // two kinds side by side in each group the sums' registers had to agree behind it: 2.64 instead of 2.58 ms for
+  // 2^20 states of 53/325, 2.51 without the signs.)
+  if (!opt.mixed) {
+    o(fmt("if (!run) { for (int q = 0; q < %d; ++q) __syncthreads(); }", (nr + GRP - 1) / GRP));
+    o("else");
+  }
+  for (bool sgn : {false, true}) {
+    o(sgn ? "else {" : "if (!sgn) {");
+    o(sums);
+    for (at = 0; at < nr; at += GRP) {
+      o("__syncthreads(); if (once) {");
+      loads();
+      for (int q = at; q < std::min(nr, at + GRP); ++q) second(q, sgn);
+      o("}");
+    }
+    o("// the sums start the float-pair accumulators");
+    for (int k = 0; k < ns; ++k) o(fmt("w[%d] = kx_mk(a%d, 0.0f);", k, k));
+    o("}");
+  }
+  o("// the warp's list of marked reactions, in class order");
   o(fmt("__shared__ short kx_lst[%d];", opt.block / 32 * (nr + 2)));
   o(fmt("short* const lst = kx_lst + (threadIdx.x >> 5) * %d;", nr + 2));
   o("const bool lead = (threadIdx.x & 31) == 0;");
@@ -2027,7 +2069,7 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
     for (int q = nw - 2; q >= 0; --q) sel = fmt("((k) < %d ? nm%d : %s)", 64 * (q + 1), q, sel.c_str());
     o("#define KX_NEG(k) ((int)((" + sel + " >> ((k) & 63)) & 1ull))");
   }
-  if (sweep) o("double Yn = Y_[i];");
+  if (sweep) o("double Yn = Y_[i];\n    float sneg = 0.0f;   // sum |Y_k|/W_k over the negative mass fractions");
   o(fmt("for (int k = 0; k < %d; ++k) {", ns));
   if (sweep) {
     o("  const double Yk = Yn;");
@@ -2043,7 +2085,7 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
   o("    if (!(l.hi > -700.0f)) l = kx_mk(-700.0f, 0.0f);");
   o("  }");
   {
-    std::string s = sweep ? "  if (__double2hiint(Yk) < 0 && yb != 0) {" : "  if (Yk < 0.0) {";
+    std::string s = sweep ? "  if (__double2hiint(Yk) < 0 && yb != 0) { sneg -= kx_d2df_i(Yk).hi * kx_iwf[2 * k];" : "  if (Yk < 0.0) {";
     for (int q = 0; q < nw; ++q) s += fmt(" %sif ((k >> 6) == %d) nm%d |= 1ull << (k & 63);", q ? "else " : "", q, q);
     o(s + " }");
   }
@@ -2534,8 +2576,8 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
     }
   };
   if (sweep) {
-    // every warp passes the sweep's barriers; a warp with a negative mass fraction skips its work and takes the
-    // class loops over all reactions, under a running scale
+    // every warp passes the sweep's barriers; a KX_FP64 warp with large negative mass fractions skips its work and
+    // takes the class loops over all reactions, under a running scale
     emit_sweep(o, g, m, cls, opt);
     o("if (in && bad) atomicMin(&kx_bad_first, (unsigned long long)i);   // a point outside the domain");
     auto write_out = [&]() {
@@ -2543,11 +2585,24 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
       o("#pragma unroll 4");
       o(fmt("for (int k = 0; k < %d; ++k) out_[(long long)k * ld + i] = bad ? KX_NAN : kx_df2d_i(w[k], S);", ns));
     };
-    if (opt.mixed) {
-      // no second copy: a state's result never depends on the states beside it
+    // the marked reactions, with signs where the warp needs them (the same arithmetic in both copies)
+    auto marked = [&](OpCounts& counts) {
+      OpCounts once;
       listed = true;
-      main_pass(c);
+      o("if (sgn) {");
+      ++o.ind;
+      main_pass(counts);
+      --o.ind;
+      o("} else {");
+      ++o.ind;
+      o("const bool anyneg = false;");
+      main_pass(once);
+      --o.ind;
+      o("}");
       write_out();
+    };
+    if (opt.mixed) {
+      marked(c);
     } else {
       o("if (!run) {");
       ++o.ind;
@@ -2558,11 +2613,8 @@ void emit_rates_class_df(Out& o, Out& g, const Mechanism& m, const EmitOptions& 
       --o.ind;
       o("} else {");
       ++o.ind;
-      o("const bool anyneg = false;");
       OpCounts once;
-      listed = true;
-      main_pass(once);
-      write_out();
+      marked(once);
       --o.ind;
       o("}");
     }

@@ -44,7 +44,7 @@ def test_against_float_pairs(name, n, precision, tmp_path):
     if n > 1:
         T[n // 2] = np.nan
     if n > 255:
-        Y[1, 40] *= -0.01     # an undershoot: its warp (mixed: the state itself) runs every reaction
+        Y[1, 40] *= -0.01     # an undershoot: its warp takes the sweep with signs
     d = to_device(torch, T, p, Y, ld=n + 3)
     w, r = (m.production_rates(*d, precision=q)[:, :n].cpu().numpy() for m, q in ((a, precision), (b, "fp64")))
     ok = np.isfinite(T)
@@ -57,8 +57,8 @@ def test_against_float_pairs(name, n, precision, tmp_path):
 @pytest.mark.parametrize("name", ["kinds", "gri_53_325"])
 @pytest.mark.parametrize("precision", ["fp64", "mixed"])
 def test_independent_of_neighbours(name, precision, tmp_path):
-    """Without an undershoot in its warp (mixed: whatever its warp holds), a state's result is the same bits
-    wherever it stands."""
+    """Without a large negative mass fraction in its warp (mixed: whatever its warp holds), a state's result is the
+    same bits wherever it stands."""
     torch = torch_cuda()
     a, _ = _pair(name, tmp_path)
     T, p, Y = _draw(name, 700, 7)
