@@ -87,9 +87,11 @@ struct EmitOptions {
 
 // Whether the production-rate kernel starts with the straight-line float32 sweep: its sums live in
 // registers, its code grows with the reactions, its marks and lists (44 bytes of marks a thread and 650 of list a
-// warp at 325 reactions) in static shared memory.  (Without reactions there is nothing to sweep.)
+// warp at 325 reactions) in static shared memory.  Without reactions there is nothing to sweep.  The no-alloc
+// kernel (opt.scratch) keeps the class loops: the sweep's sums spill to 650 bytes of local memory a thread at
+// 53/325, which the driver would back for every resident thread; the loops take 32.
 inline bool rates_swept(const Mechanism& m, const EmitOptions& opt, bool rop) {
-  return !rop && m.nr() > 0 && (opt.mixed ? opt.rates_mode == 0 : opt.rates_arith != 1 || opt.scratch) && opt.rates_negligible == 0 && m.ns <= 64 &&
+  return !rop && m.nr() > 0 && !opt.scratch && (opt.mixed ? opt.rates_mode == 0 : opt.rates_arith != 1) && opt.rates_negligible == 0 && m.ns <= 64 &&
          m.nr() <= 400 && opt.block <= 512;
 }
 

@@ -53,3 +53,14 @@ def test_inert_mixture_runs(tmp_path):
             assert torch.count_nonzero(h.production_rates(T, p, Y, precision=precision)) == 0
         for a, b in zip(h.thermo(T, p, Y) + h.transport(T, p, Y), full.thermo(T, p, Y) + full.transport(T, p, Y)):
             assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("name,most", [("h2o2_9_21", 32), ("gri_53_325", 64), ("53_400", 64)])
+def test_noalloc_kernel_keeps_its_vectors_in_the_scratch(name, most, tmp_path):
+    """Almost no local memory per thread, which the driver would back for every resident thread of the device:
+    32 bytes at 53/325, 24 at 53 species and 400 reactions."""
+    m = copy.deepcopy(synth.mechanism("gri_53_325" if name == "53_400" else name))
+    if name == "53_400":
+        m.reactions = m.reactions + m.reactions[:75]
+    k = _compile(m, tmp_path / "m.kxmech", ("wdot_fp64_noalloc",))
+    assert k["wdot_fp64_noalloc"]["local_bytes"] <= most
