@@ -15,7 +15,11 @@
 // below 2^24 are exact there, so the levels carry the 50-bit fixed-point
 // product without rounding (the splitting scheme of Ozaki et al., Numer.
 // Algorithms 59 (2012), on float16 units as in Mukunoki et al., ISC 2020),
-// and the kernel adds the levels up in float pairs.  A coefficient set whose
+// and the kernel adds the levels up in float pairs.  The first level's sum is
+// 2^18 sum v c, and those after it add products of lower digits, whose signs
+// are as good as random: with sum v c <= kSumMost a level stays below 0.9 x 2^24
+// for states of like mass fractions too.  53/325's rows reach sum |c| = 33.7;
+// 160/900's 108, and there a state's v are halved until sum v <= kSumMost.  A coefficient set whose
 // basis function is scaled by 2^E_m takes (50 + E_m)/10 digits.  Mixed
 // precision takes digits up to 2^-27 and adds the levels in float32.
 //
@@ -212,6 +216,7 @@ constexpr int kPhiE = -30;                // ... by 2^-30 or less evaluated in f
                                          // rounded t is off by 2^-16 (t = +-1) to 2^-20 of itself
 constexpr int kMidE = -14;                // ... by 2^-14 or less with one exact product
 constexpr int kDigit = 10;                 // bits of a digit
+constexpr int kSumMost = 40;               // largest sum v c of a row and basis function
 constexpr int kStates = 128, kRowsChunk = 16, kGroups = 4;   // states a tile; rows a chunk; groups of 128 compute threads
 
 struct Stage {
@@ -227,6 +232,7 @@ struct Stage {
 struct Plan {
   TcBasis b;
   bool mixed = false;
+  bool bound_v = false;                    // some row's sum |c| exceeds kSumMost
   int part = 1;
   int nd = 5;                              // digits of v
   std::vector<int> lev;                    // digits (and levels) of basis function m
@@ -245,6 +251,12 @@ bool make_plan(const Mechanism& m, const EmitOptions& opt, Plan& p) {
   if (opt.part == 3 ? !tc_thermo(m, p.b, p.mids) : !tc_basis(m, opt.part, opt.mixed, p.b)) return false;
   const TcBasis& b = p.b;
   p.nd = opt.mixed ? 3 : 5;
+  for (int r = 0; r < b.rows; ++r)
+    for (int q = 0; q <= b.M; ++q) {
+      double sum = 0;
+      for (int j = 0; j < b.ns; ++j) sum += std::fabs(b.coef[((size_t)r * b.ns + j) * (b.M + 1) + q]);
+      p.bound_v |= !opt.mixed && sum > kSumMost;   // (mixed: float32's rounding is what it allows)
+    }
   // digits that keep each set's dropped products near 2^-48 of the largest v (mixed: 2^-26)
   const double bits = opt.mixed ? 26.0 : 50.0;
   p.lev.resize(b.M + 1);
@@ -713,7 +725,21 @@ std::string emit_transport_tc(const Mechanism& m, const EmitOptions& opt, const 
     << "      KX_COMPUTE_SYNC;\n"   // (the previous tile's shared values are no longer read)
     << "      #pragma unroll\n"
     << "      for (int q = 0; q < " << G << "; ++q) mx = max(mx, __float_as_int(sred[q * 128 + s].x));\n"
-    << "      if (mx >= 100000 || mx < 64) gen = true;\n"
+    << "      if (mx >= 100000 || mx < 64) gen = true;\n";
+  if (p.bound_v) {
+    // sum v in units of 2^-12 from the mantissas' first 12 bits (rounded up), over the compute groups
+    s << "      int sv = 0;\n"
+      << "      #pragma unroll 4\n"
+      << fmt("      for (int q = 0; q < %d; ++q) {\n", 4 * QW)
+      << fmt("        const int j = wg * %d + q;\n", 4 * QW)
+      << "        const int hi = __double2hiint(" << yval("j") << ");\n"
+      << "        sv += (int)((0x801u + (((unsigned)hi >> 9) & 0x7ffu)) >> min((unsigned)(mx - sec[j] - ((hi >> 20) & 0x7ff)), 31u));\n      }\n"
+      << "      sred[wg * 128 + s].y = __int_as_float(sv);\n      KX_COMPUTE_SYNC;\n      sv = 0;\n"
+      << "      #pragma unroll\n"
+      << "      for (int q = 0; q < " << G << "; ++q) sv += __float_as_int(sred[q * 128 + s].y);\n"
+      << fmt("      for (int most = %d; sv > most && most < %d; most *= 2) ++mx;\n", kSumMost * 4096, 4096 * ns);
+  }
+  s
     << "      const bool off = bad || gen;\n"
     << "      const int sc = off ? 0 : 1022 - mx;   // v_j = Y_j 2^(ecol_j + sc), the largest in [1/2, 1)\n"
     << "      if (off) mx = 1 << 20;\n";

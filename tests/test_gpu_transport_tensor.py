@@ -122,3 +122,30 @@ def test_same_bits_alone_and_in_a_batch(precision):
         part = mech.transport(T[a:b].contiguous(), p[a:b].contiguous(), Y[:, a:b].contiguous(), precision=precision)
         for x, y in zip(part, whole):
             assert torch.equal(x, y[..., a:b])
+
+
+@pytest.mark.parametrize("kernel", ["visc_fp64", "diff_fp64", "thermo"])
+@pytest.mark.parametrize("name", ["gri_53_325", "large_160_900"])
+def test_like_mass_fractions(name, kernel):
+    """All of a kernel's scaled mass fractions near their largest: the largest sums that its products' exact integer
+    accumulation has to hold (108 of the 64 that float32 holds, for a row of 160/900's viscosity)."""
+    import re
+    torch = torch_cuda()
+    mech = mechanism(name)
+    src = mech.kernel_source(kernel)
+    ecol = np.array([int(v) for v in re.search(r"kx_ecol\[\d+\] = \{(.*?)\}", src).group(1).split(",") if v.strip()])
+    T, p, Y = states(name, 256)
+    rng = np.random.default_rng(2)
+    u = 1.0 - rng.uniform(0.0, 0.02, Y.shape) * (np.arange(256) % 2)        # every other state: all alike
+    Y = u * 2.0 ** -(ecol[:Y.shape[0], None] + 8.0)                        # the products' v: u (unnormalised states)
+    d = to_device(torch, T, p, Y)
+    if kernel == "thermo":
+        got, ref = mech.thermo(*d), oracle(name).thermo(T, p, Y)
+        ref = (ref[0], ref[1])
+    else:
+        got, ref = mech.transport(*d), oracle(name).transport(T, p, Y)
+        got, ref = (got[:2], ref[:2]) if kernel == "visc_fp64" else (got[2:], ref[2:])
+    for a, b in zip(got, ref):
+        a = a.cpu().numpy()
+        err = np.abs(a - b) / (np.abs(b) if kernel != "thermo" else np.abs(b).max())
+        assert err.max() <= 1e-13, f"{err.max():.2e}"
