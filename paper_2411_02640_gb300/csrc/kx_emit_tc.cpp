@@ -609,6 +609,8 @@ std::string emit_transport_tc(const Mechanism& m, const EmitOptions& opt, const 
     << "double* __restrict__ out0_, double* __restrict__ out1_, " << (thermo ? "" : "double* __restrict__ out2_, ") << "long long n)\n{\n";
   s << "  __shared__ __align__(8) unsigned long long bars[" << 2 * p.slots + 5 << "];\n";
   s << "  __shared__ unsigned tmem_addr;\n";
+  // a compute warp whose wait ran out says so to the groups that read its shared values
+  s << "  __shared__ volatile int failed;\n";
   s << "  kx_load_tables();\n";
   s << "  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;\n";
   s << "  unsigned char* const slots = kx_dyn;\n";
@@ -627,7 +629,7 @@ std::string emit_transport_tc(const Mechanism& m, const EmitOptions& opt, const 
   s << "  if (threadIdx.x == 0) {\n"
     << "    for (int j = 0; j < " << p.slots << "; ++j) { kx_mb_init(full + 8 * j, 1); kx_mb_init(empty + 8 * j, 1); }\n"
     << "    for (int j = 0; j < 2; ++j) { kx_mb_init(dfull + 8 * j, 1); kx_mb_init(dfree + 8 * j, " << 4 * G << "); }\n"
-    << "    kx_mb_init(aready, " << 4 * G << ");\n"
+    << "    kx_mb_init(aready, " << 4 * G << ");\n    failed = 0;\n"
     << "    asm volatile(\"fence.mbarrier_init.release.cluster;\" ::: \"memory\");\n"
     << "  }\n";
   s << fmt("  if (warp == %d) {\n", 4 * G)
@@ -707,6 +709,7 @@ std::string emit_transport_tc(const Mechanism& m, const EmitOptions& opt, const 
     << "      const bool in = t * 128 + s < n;\n"
     << "      bool bad = !(T > 0.0 && P > 0.0 && T < KX_INF && P < KX_INF);\n"
     << (thermo ? std::string("      bool gen = false;\n") : fmt("      bool gen = !(T >= %s && T <= %s);\n", D(kTcTlo).c_str(), D(kTcThi).c_str()));
+  const char* kShare = "if (!ok) failed = 1;\n      KX_COMPUTE_SYNC;\n      ok = __all_sync(0xffffffffu, ok && !failed);\n";
   auto yval = [&](const std::string& j) {
     return stage_y ? fmt("sy[(%s) * 128 + s]", j.c_str()) : fmt("((%s) < %d ? Y_[(long long)(%s) * ld + i] : 0.0)", j.c_str(), ns, j.c_str());
   };
@@ -872,9 +875,9 @@ std::string emit_transport_tc(const Mechanism& m, const EmitOptions& opt, const 
   const char* LO = mixed ? "0.0f" : "lo[a]";
   if (thermo) {
     s << fmt("      #pragma unroll\n      for (int a = 0; a < %d; ++a) sred[(8 + c * 16 + wg * %d + a) * 128 + s] = make_float2(hi[a], lo[a]);\n      }\n", RT, RT)
-      << "      KX_COMPUTE_SYNC;\n"
+      << "      " << kShare
       // c_p = sum B_n x^n, h = h(x = 0) + T_half x sum B_n/(n + 1) x^n over the T_mid groups
-      << "      if (wg < 2 && in && !bad && !gen) {\n"
+      << "      if (wg < 2 && in && !bad && !gen && ok) {\n"
       << "        const kx_df Td = kx_d2df_i(T);\n        kx_df v = kx_mk(0.0f, 0.0f);\n";
     for (size_t g = 0; g < p.mids.size(); ++g) {
       long long bits;
@@ -902,7 +905,7 @@ std::string emit_transport_tc(const Mechanism& m, const EmitOptions& opt, const 
   } else {
   s << "      if (c == 0) {\n"
     << fmt("        #pragma unroll\n        for (int a = 0; a < %d; ++a)\n          if (wg * %d + a < %d) sred[(8 + wg * %d + a) * 128 + s] = make_float2(hi[a], %s);\n", RT, RT, b.first, RT, LO)
-    << "        KX_COMPUTE_SYNC;\n"
+    << "        " << kShare
     << "        const float2 c0 = sred[8 * 128 + s], c1 = sred[9 * 128 + s], g0 = sred[4 * 128 + s];\n"
     << "        if (!gen && !(c0.x > 0.0f)) bad = true;\n";
   if (diff) {
@@ -913,7 +916,7 @@ std::string emit_transport_tc(const Mechanism& m, const EmitOptions& opt, const 
     else
       s << "        sYs = c1.x;\n        fac = __fdividef(c0.x, c1.x) * __fdividef(" << F(P_ATM) << ", kx_d2f(P)) / g0.x;\n";
   } else {
-    s << "        if (wg == 0 && in && !bad && !gen) {\n"
+    s << "        if (wg == 0 && in && !bad && !gen && ok) {\n"
       << "          const float2 c2 = sred[10 * 128 + s], c3 = sred[11 * 128 + s], c4 = sred[12 * 128 + s], g1 = sred[5 * 128 + s];\n";
     // sum X lambda = g1 (c1 + c3)/c0, sum X/lambda = (c2 + c4)/(c0 g1), each row under its own power of two
     auto sum2 = [&](const char* x, int rx, const char* y, int ry) {
@@ -940,7 +943,7 @@ std::string emit_transport_tc(const Mechanism& m, const EmitOptions& opt, const 
   s << "      }\n";
   // this chunk's rows
   s << "      if (c != 0 || cy == 0) {\n"
-    << "        const bool act = in && !bad && !gen;\n"
+    << "        const bool act = in && !bad && !gen && ok;\n"
     << fmt("        const int k0 = c * 16 + wg * %d - %d;   // the first row's species (the same in every lane)\n", RT, b.first);
   if (visc) {
     s << fmt("        #pragma unroll\n        for (int a = 0; a < %d; ++a) {\n", RT)
@@ -979,8 +982,8 @@ std::string emit_transport_tc(const Mechanism& m, const EmitOptions& opt, const 
   }
   s << "      }\n      }\n";
   if (visc) {
-    s << "      sred[(16 + wg) * 128 + s] = make_float2(mu.hi, mu.lo);\n      KX_COMPUTE_SYNC;\n"
-      << "      if (wg == 0 && in && !bad && !gen) {\n"
+    s << "      sred[(16 + wg) * 128 + s] = make_float2(mu.hi, mu.lo);\n      " << kShare
+      << "      if (wg == 0 && in && !bad && !gen && ok) {\n"
       << "        const float2 g0 = sred[4 * 128 + s];\n";
     if (!mixed)
       s << "        for (int w = 1; w < " << G << "; ++w) { const float2 v = sred[(16 + w) * 128 + s]; mu = kx_df_add(mu, kx_mk(v.x, v.y)); }\n"
@@ -992,8 +995,18 @@ std::string emit_transport_tc(const Mechanism& m, const EmitOptions& opt, const 
   }
   }
   // states outside the domain, outside the basis' temperatures or with non-finite mass fractions
-  s << "      if (cy == 0 && __any_sync(0xffffffffu, in && (bad || gen || !ok))) {\n"
-    << "        bad = bad || !ok;\n";
+  // A wait that ran out: every block's own results are nan, and the point recorded (diffusion: the rows of this
+  // warp's group in the block's chunks; else by the group that writes them, which has seen the others' flag)
+  s << "      if (!ok && in) {\n"
+    << (diff ? "        atomicMin(&kx_bad_first, (unsigned long long)i);\n" : "        if (wg == 0) atomicMin(&kx_bad_first, (unsigned long long)i);\n");
+  if (diff)
+    s << fmt("        for (int c = cy; c < %d; c += gy)\n          for (int a = 0; a < %d; ++a) {\n", p.chunks, RT)
+      << fmt("            const int k = c * 16 + wg * %d + a - %d;\n", RT, b.first)
+      << fmt("            if (k >= 0 && k < %d) out2_[(long long)k * ld + i] = KX_NAN;\n          }\n", ns);
+  else
+    s << "        if (wg == 0) { out0_[i] = KX_NAN; out1_[i] = KX_NAN; }\n";
+  s << "      }\n";
+  s << "      if (cy == 0 && ok && __any_sync(0xffffffffu, in && (bad || gen))) {\n";
   if (!thermo)
     s << "        double isig = 0.0;\n"
       << "        if (!bad) {\n"
