@@ -216,7 +216,10 @@ kx_status kx_thermo(kx_handle h, const double* T, const double* p, const double*
  * ln eta_k, ln lambda_k and ln D_kj (Sec. A.3.4), D_kj scaled by p_atm/p.
  * A species whose partners all have X_j = 0 gets its self-diffusion D_kk.
  * The default kernels hold the fits' temperature dependence for 200 to 4000 K;
- * states outside are evaluated pair by pair (slower, the same accuracy). */
+ * states outside are evaluated pair by pair, at the same accuracy: where they
+ * are a few per cent of a batch about twice its time (2^18 states of 53
+ * species: 1.4 ms with 1 % outside, 0.7 with none, 3.2 with tr_layout = 3),
+ * where they are all of it tr_layout = 3 is two to five times faster. */
 kx_status kx_transport(kx_handle h, const double* T, const double* p, const double* Y, int64_t ld,
                        double* mu, double* lambda, double* Dk, int64_t n, kx_precision precision, void* stream);
 

@@ -57,6 +57,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <functional>
 
 #include "kx_emit_text.h"
 #include "kx_internal.h"
@@ -381,25 +382,51 @@ void emit_pairwise(std::ostringstream& s, const Mechanism& m, const Plan& p) {
   for (int k = 0; k < ns; ++k) { iw[k] = 1.0 / m.W[k]; w[k] = m.W[k]; }
   s << "__device__ const double kx_iw[" << ns << "] = {" << list(iw, false) << "};\n";
   s << "__device__ const double kx_w[" << ns << "] = {" << list(w, false) << "};\n";
-  auto horner = [](const char* tab) {
-    return fmt("kx_df_fma_u(kx_df_fma_u(kx_df_fma_u(kx_df_fma_u(kx_f2(%s[4]), L, kx_f2(%s[3])), L, kx_f2(%s[2])), L, kx_f2(%s[1])), L, "
-               "kx_f2(%s[0]))", tab, tab, tab, tab, tab);
+  // degree-4 polynomial in L whose coefficient n of a warp's lanes is the expression tab(n)
+  auto horner = [](const std::function<std::string(int)>& tab) {
+    std::string e = tab(4);
+    for (int n = 3; n >= 0; --n) e = fmt("kx_df_fma_u(%s, L, %s)", e.c_str(), tab(n).c_str());
+    return e;
   };
+  const int SL = (ns + 31) / 32;   // species of a lane: lane, lane + 32, ...
+  const std::string last = std::to_string(ns - 1);
   s << "__device__ __forceinline__ kx_df kx_f2(float2 v) { return kx_mk(v.x, v.y); }\n";
+  if (p.part != 3)
+    s << "__device__ __forceinline__ double kx_lane_sum(double v) {\n"
+      << "  for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);\n  return v;\n}\n"
+      << "__device__ __forceinline__ kx_df kx_lane_sum(kx_df v) {\n"
+      << "  for (int d = 16; d > 0; d >>= 1) v = kx_df_add(v, kx_mk(__shfl_xor_sync(0xffffffffu, v.hi, d), __shfl_xor_sync(0xffffffffu, v.lo, d)));\n"
+      << "  return v;\n}\n";
+  // chains that a warp of the state functions below has in flight (SL rows of a lane, as many species at a time)
+  const int unroll = std::max(1, 4 / SL);
   if (p.part == 2) {
-    std::vector<double> dc, ds;
+    // -ln D_jk about L_mid, coefficient n of (j, k) at (n ns + j) ns + k: a warp's lanes (k, or j: it is symmetric)
+    // read 32 neighbours
+    std::vector<unsigned long long> dc(5 * (size_t)ns * ns);
     for (int k = 0; k < ns; ++k)
       for (int j = k; j < ns; ++j) {
         double d[5];
         shift_poly(&m.dif[5 * ((size_t)k * ns + j)], kTcLmid, -1.0, d);
-        for (int n = 0; n < 5; ++n) dc.push_back(d[n]);
+        for (int n = 0; n < 5; ++n) {
+          const float h = (float)d[n], l = (float)(d[n] - (double)h);
+          unsigned hb, lb;
+          std::memcpy(&hb, &h, 4);
+          std::memcpy(&lb, &l, 4);
+          dc[((size_t)n * ns + j) * ns + k] = dc[((size_t)n * ns + k) * ns + j] = (unsigned long long)lb << 32 | hb;
+        }
       }
-    s << "__device__ const float2 kx_dc[" << dc.size() << "] = {" << list(dc, true) << "};\n";
+    s << "__device__ const unsigned long long kx_dcb[" << dc.size() << "] = {";
+    for (unsigned long long v : dc) s << hex64(v) << ",";
+    s << "};\n";
+    s << "__device__ __forceinline__ kx_df kx_dc(int n, int j, int k) {\n"
+      << fmt("  const unsigned long long b = kx_dcb[(n * %d + j) * %d + k];\n", ns, ns)
+      << "  return kx_mk(__uint_as_float((unsigned)b), __uint_as_float((unsigned)(b >> 32)));\n}\n";
+    auto coef = [](const char* j, const char* k) {
+      return [=](int n) { return fmt("kx_dc(%d, %s, %s)", n, j, k); };
+    };
     // D_k of state i by one warp, its lanes over the partner species: the partners' share of the mass
     // summed directly, so that a nearly pure state keeps its relative accuracy; D_kk where no partner is
     // present.  Every lane returns the value (sums in a fixed order).
-    s << "__device__ __forceinline__ double kx_lane_sum(double v) {\n"
-      << "  for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);\n  return v;\n}\n";
     s << "__device__ __noinline__ double kx_diff_row(const double* __restrict__ Y_, long long ld, long long i, int k, float Lh, float Ll, double P) {\n"
       << "  const int lane = threadIdx.x & 31;\n  const kx_df L = kx_mk(Lh, Ll);\n"
       << "  double sy = 0.0, sY = 0.0, so = 0.0;\n"
@@ -409,15 +436,64 @@ void emit_pairwise(std::ostringstream& s, const Mechanism& m, const Plan& p) {
       << "  kx_df S = kx_mk(0.f, 0.f);\n"
       << "  for (int j = lane; j < " << ns << "; j += 32) {\n"
       << "    if (j == k) continue;\n"
-      << "    const int a = min(j, k), c = max(j, k);\n"
-      << "    const float2* t = kx_dc + 5 * (a * " << ns << " - a * (a - 1) / 2 + c - a);\n"
-      << "    S = kx_df_fma_u(kx_d2df_i(Y_[(long long)j * ld + i] * kx_iw[j] * isig), kx_df_exp(" << horner("t") << "), S);\n"
+      << "    S = kx_df_fma_u(kx_d2df_i(Y_[(long long)j * ld + i] * kx_iw[j] * isig), kx_df_exp(" << horner(coef("k", "j")) << "), S);\n"
       << "  }\n"
       << "  const double Sd = kx_lane_sum(kx_df2d(kx_df_norm(S))), pr = " << D(P_ATM) << " / P;\n"
       << "  if (Sd > 0.0) return so / sY * pr / Sd;\n"
-      << "  const float2* t = kx_dc + 5 * (k * " << ns << " - k * (k - 1) / 2);\n"
-      << "  const kx_df e = " << horner("t") << ";\n"
+      << "  const kx_df e = " << horner(coef("k", "k")) << ";\n"
       << "  return kx_df2d(kx_df_exp(kx_mk(-e.hi, -e.lo))) * pr;\n}\n";
+    // All D_k of state i by one warp, its lanes over the rows, every species' mole fraction broadcast to them in turn.
+    // 2^18 states of 53/325 at 4500 K: 6.5 ms (mixed 2.7), a row at a time as above 58; with 1 % of them there 0.84
+    // against 1.82, with none 0.30.  Bound by the coefficients' way from L2 (40 bytes a pair) and the latency of
+    // four warps a scheduler; the one-thread-per-state kernel, which a call cannot know to choose, takes 1.8.
+    if (p.mixed)   // 1/D_jk to about 2^-22: the polynomial's last sum and the exponential's argument in two parts
+      s << "__device__ __forceinline__ float kx_idiff(int j, int k, float L) {\n"
+        << "  const float h = fmaf(fmaf(fmaf(kx_dc(4, j, k).hi, L, kx_dc(3, j, k).hi), L, kx_dc(2, j, k).hi), L, kx_dc(1, j, k).hi);\n"
+        << "  const kx_df c = kx_dc(0, j, k);\n"
+        << "  const float p = __fmul_rn(h, L);\n"
+        << "  const kx_df e = kx_ts(c.hi, p);\n"
+        << "  const float lo = e.lo + (fmaf(h, L, -p) + c.lo), y = __fmul_rn(e.hi, 1.44269504f);\n"
+        << "  const float yl = fmaf(e.hi, 1.44269504f, -y) + fmaf(e.hi, 1.92596303e-8f, lo * 1.44269504f);\n"
+        << "  float r;\n  asm(\"ex2.approx.ftz.f32 %0, %1;\" : \"=f\"(r) : \"f\"(y));\n"
+        << "  return fmaf(r, yl * 0.693147181f, r);\n}\n";
+    s << "__device__ __noinline__ void kx_diff_state(const double* __restrict__ Y_, long long ld, long long i, float Lh, float Ll, double P, double* __restrict__ out) {\n"
+      << "  const int lane = threadIdx.x & 31;\n  const kx_df L = kx_mk(Lh, Ll);\n"
+      << fmt("  double y[%d], so[%d], sy = 0.0, sY = 0.0;\n", SL, SL)
+      << fmt("  #pragma unroll\n  for (int s = 0; s < %d; ++s) {\n", SL)
+      << fmt("    const int k = lane + 32 * s;\n    y[s] = k < %d ? Y_[(long long)k * ld + i] : 0.0;\n", ns)
+      << "    sY += y[s]; sy = fma(y[s], kx_iw[min(k, " << last << ")], sy);\n  }\n"
+      << "  sy = kx_lane_sum(sy); sY = kx_lane_sum(sY);\n"
+      << "  const double isig = 1.0 / sy;\n"
+      << "  if (!(isig > 0.0 && isig < KX_INF)) {   // outside the domain\n"
+      << fmt("    for (int k = lane; k < %d; k += 32) out[(long long)k * ld + i] = KX_NAN;\n", ns)
+      << "    if (lane == 0) atomicMin(&kx_bad_first, (unsigned long long)i);\n    return;\n  }\n"
+      << (p.mixed ? fmt("  float x[%d], S[%d];\n", SL, SL) : fmt("  kx_df x[%d], S[%d];\n", SL, SL))
+      << fmt("  #pragma unroll\n  for (int s = 0; s < %d; ++s) {\n", SL)
+      << "    const kx_df X = kx_d2df_i(y[s] * kx_iw[min(lane + 32 * s, " << last << ")] * isig);\n"
+      << (p.mixed ? "    x[s] = X.hi; S[s] = 0.0f;\n" : "    x[s] = X; S[s] = kx_mk(0.0f, 0.0f);\n")
+      // the partners' share of the mass: the rest of the sum, for a species of more than half of it summed directly
+      << "    so[s] = sY - y[s];\n"
+      << "    for (unsigned m = __ballot_sync(0xffffffffu, y[s] > 0.5 * sY); m; m &= m - 1) {\n"
+      << "      const bool own = lane == __ffs(m) - 1;\n      double d = 0.0;\n"
+      << fmt("      #pragma unroll\n      for (int q = 0; q < %d; ++q) if (!own || q != s) d += y[q];\n", SL)
+      << "      d = kx_lane_sum(d);\n      if (own) so[s] = d;\n    }\n  }\n"
+      << fmt("  #pragma unroll\n  for (int q = 0; q < %d; ++q)\n    #pragma unroll %d\n", SL, unroll)
+      << fmt("    for (int jl = 0; jl < min(32, %d - 32 * q); ++jl) {\n      const int j = 32 * q + jl;\n", ns)
+      << (p.mixed ? "      const float xj = __shfl_sync(0xffffffffu, x[q], jl);\n"
+                  : "      const kx_df xj = kx_mk(__shfl_sync(0xffffffffu, x[q].hi, jl), __shfl_sync(0xffffffffu, x[q].lo, jl));\n")
+      << fmt("      #pragma unroll\n      for (int s = 0; s < %d; ++s) {\n", SL)
+      << "        const int k = min(lane + 32 * s, " << last << ");\n"
+      << (p.mixed ? "        S[s] = fmaf(k == j ? 0.0f : xj, kx_idiff(j, k, Lh), S[s]);\n"
+                  : "        S[s] = kx_df_fma_u(k == j ? kx_mk(0.0f, 0.0f) : xj, kx_df_exp(" + horner(coef("j", "k")) + "), S[s]);\n")
+      << "      }\n    }\n"
+      << "  const double pr = " << D(P_ATM) << " / P;\n"
+      << fmt("  #pragma unroll\n  for (int s = 0; s < %d; ++s) {\n", SL)
+      << fmt("    const int k = lane + 32 * s;\n    if (k >= %d) break;\n", ns)
+      << (p.mixed ? "    const double Sd = kx_f2d(S[s]);\n" : "    const double Sd = kx_df2d(kx_df_norm(S[s]));\n")
+      << "    double d = so[s] * pr / (sY * Sd);\n"
+      << "    if (!(Sd > 0.0)) {\n      const kx_df e = " << horner(coef("k", "k")) << ";\n"
+      << "      d = kx_df2d(kx_df_exp(kx_mk(-e.hi, -e.lo))) * pr;\n    }\n"
+      << "    out[(long long)k * ld + i] = d;\n  }\n}\n";
     return;
   }
   if (p.part == 3) {
@@ -437,6 +513,7 @@ void emit_pairwise(std::ostringstream& s, const Mechanism& m, const Plan& p) {
       << "  }\n  return make_double2(cp, h);\n}\n";
     return;
   }
+  // u_k = sqrt(eta_k) W_k^(-1/4), v = 1/u: sum_j X_j phi_kj = sum_j a_kj X_j (1 + u_k v_j)^2, a_kj at j ns + k
   std::vector<double> pv, pl, wa, sq;
   for (int k = 0; k < ns; ++k) {
     double d[5];
@@ -445,36 +522,56 @@ void emit_pairwise(std::ostringstream& s, const Mechanism& m, const Plan& p) {
     for (int n = 0; n < 5; ++n) pv.push_back(d[n]);
     shift_poly(&m.lam[5 * k], kTcLmid, 1.0, d);
     for (int n = 0; n < 5; ++n) pl.push_back(d[n]);
-    for (int j = 0; j < ns; ++j) wa.push_back(1.0 / std::sqrt(8.0 * (1.0 + m.W[k] / m.W[j])));
+    for (int j = 0; j < ns; ++j) wa.push_back(1.0 / std::sqrt(8.0 * (1.0 + m.W[j] / m.W[k])));
     sq.push_back(std::sqrt(m.W[k]));
   }
   s << "__device__ const float2 kx_pv[" << pv.size() << "] = {" << list(pv, true) << "};\n";
   s << "__device__ const float2 kx_pl[" << pl.size() << "] = {" << list(pl, true) << "};\n";
   s << "__device__ const float2 kx_wa[" << wa.size() << "] = {" << list(wa, true) << "};\n";
-  s << "__device__ const double kx_sqw[" << ns << "] = {" << list(sq, false) << "};\n";
-  // u_k = sqrt(eta_k) W_k^(-1/4), v = 1/u: sum_j X_j phi_kj = sum_j a_kj X_j (1 + u_k v_j)^2
-  s << "__device__ __noinline__ double2 kx_visc_state(const double* __restrict__ Y_, long long ld, long long i, kx_df L, double isig) {\n"
-    << "  float2 x[" << ns << "], v[" << ns << "];\n"
-    << "  kx_df sl = kx_mk(0.f, 0.f), sil = kx_mk(0.f, 0.f);\n"
-    << "  for (int k = 0; k < " << ns << "; ++k) {\n"
-    << "    const kx_df X = kx_d2df_i(Y_[(long long)k * ld + i] * kx_iw[k] * isig);\n"
+  s << "__device__ const float2 kx_sqw[" << ns << "] = {" << list(sq, true) << "};\n";
+  auto of = [](const char* t) { return [=](int n) { return fmt("kx_f2(%s[%d])", t, n); }; };
+  // mu and lambda of state i by one warp, its lanes over Wilke's rows, every species' mole fraction and v broadcast
+  // to them in turn.  2^18 states of 53/325 at 4500 K: 2.4 ms (mixed 1.6), with a thread for each state 4.4; with 1 %
+  // of them there 0.59 against 4.1, with none 0.36; the one-thread-per-state kernel takes 1.3.
+  s << "__device__ __noinline__ double2 kx_visc_state(const double* __restrict__ Y_, long long ld, long long i, float Lh, float Ll) {\n"
+    << "  const int lane = threadIdx.x & 31;\n  const kx_df L = kx_mk(Lh, Ll);\n"
+    << (p.mixed ? fmt("  float x[%d], u[%d], v[%d], S[%d];\n", SL, SL, SL, SL) : fmt("  kx_df x[%d], u[%d], v[%d], S[%d];\n", SL, SL, SL, SL))
+    << fmt("  double y[%d], sy = 0.0;\n  kx_df w[%d], sl = kx_mk(0.f, 0.f), sil = kx_mk(0.f, 0.f);\n", SL, SL)
+    << fmt("  #pragma unroll\n  for (int s = 0; s < %d; ++s) {\n", SL)
+    << "    const int k = min(lane + 32 * s, " << last << ");\n"
+    << fmt("    y[s] = lane + 32 * s < %d ? Y_[(long long)k * ld + i] * kx_iw[k] : 0.0;\n    sy += y[s];\n  }\n", ns)
+    << "  const double isig = 1.0 / kx_lane_sum(sy);\n"
+    << "  if (!(isig > 0.0 && isig < KX_INF)) {   // outside the domain\n"
+    << "    if (lane == 0) atomicMin(&kx_bad_first, (unsigned long long)i);\n    return make_double2(KX_NAN, KX_NAN);\n  }\n"
+    << fmt("  #pragma unroll\n  for (int s = 0; s < %d; ++s) {\n", SL)
+    << "    const int k = min(lane + 32 * s, " << last << ");\n"
+    << "    const kx_df X = kx_d2df_i(y[s] * isig);\n"
     << "    const float2* pv = kx_pv + 5 * k; const float2* pl = kx_pl + 5 * k;\n"
-    << "    const kx_df e = kx_df_exp(" << horner("pv") << "), l = " << horner("pl") << ";\n"
-    << "    x[k] = make_float2(X.hi, X.lo); v[k] = make_float2(e.hi, e.lo);\n"
+    << "    const kx_df e = " << horner(of("pv")) << ", l = " << horner(of("pl")) << ";\n"
+    << "    const kx_df ve = kx_df_exp(e), ue = kx_df_exp(kx_mk(-e.hi, -e.lo));\n"
+    << (p.mixed ? "    x[s] = X.hi; v[s] = ve.hi; u[s] = ue.hi; S[s] = 0.0f;\n" : "    x[s] = X; v[s] = ve; u[s] = ue; S[s] = kx_mk(0.f, 0.f);\n")
+    << "    w[s] = kx_df_mul(X, kx_df_mul(kx_df_mul(ue, ue), kx_f2(kx_sqw[k])));\n"
     << "    sl = kx_df_fma(X, kx_df_exp(l), sl); sil = kx_df_fma(X, kx_df_exp(kx_mk(-l.hi, -l.lo)), sil);\n"
     << "  }\n"
-    << "  double mu = 0.0;\n"
-    << "  for (int k = 0; k < " << ns << "; ++k) {\n"
-    << "    const float2* pv = kx_pv + 5 * k;\n"
-    << "    const kx_df e = " << horner("pv") << ", u = kx_df_exp(kx_mk(-e.hi, -e.lo));\n"
-    << "    kx_df s = kx_mk(0.f, 0.f);\n"
-    << "    for (int j = 0; j < " << ns << "; ++j) {\n"
-    << "      const kx_df w = kx_df_fma_u(u, kx_f2(v[j]), kx_mk(1.f, 0.f));\n"
-    << "      s = kx_df_fma_u(kx_df_mul_u(kx_f2(kx_wa[k * " << ns << " + j]), kx_f2(x[j])), kx_df_mul_u(w, w), s);\n"
-    << "    }\n"
-    << "    mu = fma(kx_df2d(kx_f2(x[k])) * kx_df2d(kx_df_mul(u, u)), kx_sqw[k] / kx_df2d(s), mu);\n"
-    << "  }\n"
-    << "  return make_double2(mu, 0.5 * (kx_df2d(sl) + 1.0 / kx_df2d(sil)));\n}\n";
+    << fmt("  #pragma unroll\n  for (int q = 0; q < %d; ++q)\n    #pragma unroll %d\n", SL, unroll)
+    << fmt("    for (int jl = 0; jl < min(32, %d - 32 * q); ++jl) {\n", ns);
+  if (p.mixed)
+    s << "      const float xj = __shfl_sync(0xffffffffu, x[q], jl), vj = __shfl_sync(0xffffffffu, v[q], jl);\n";
+  else
+    s << "      const kx_df xj = kx_mk(__shfl_sync(0xffffffffu, x[q].hi, jl), __shfl_sync(0xffffffffu, x[q].lo, jl));\n"
+      << "      const kx_df vj = kx_mk(__shfl_sync(0xffffffffu, v[q].hi, jl), __shfl_sync(0xffffffffu, v[q].lo, jl));\n";
+  s << fmt("      #pragma unroll\n      for (int s = 0; s < %d; ++s) {\n", SL)
+    << fmt("        const float2 a = kx_wa[(32 * q + jl) * %d + min(lane + 32 * s, %s)];\n", ns, last.c_str());
+  if (p.mixed)
+    s << "        const float z = fmaf(u[s], vj, 1.0f);\n        S[s] = fmaf(a.x * xj, z * z, S[s]);\n";
+  else
+    s << "        const kx_df z = kx_df_fma_u(u[s], vj, kx_mk(1.f, 0.f));\n"
+      << "        S[s] = kx_df_fma_u(kx_df_mul_u(kx_f2(a), xj), kx_df_mul_u(z, z), S[s]);\n";
+  s << "      }\n    }\n  kx_df mu = kx_mk(0.f, 0.f);\n"
+    << fmt("  #pragma unroll\n  for (int s = 0; s < %d; ++s) mu = kx_df_add(mu, kx_df_div(w[s], ", SL)
+    << (p.mixed ? "kx_mk(S[s], 0.0f)));\n" : "kx_df_norm(S[s])));\n")
+    << "  mu = kx_lane_sum(mu); sl = kx_lane_sum(sl); sil = kx_lane_sum(sil);\n"
+    << "  return make_double2(kx_df2d(mu), 0.5 * kx_df2d(kx_df_add(sl, kx_df_div(kx_mk(1.0f, 0.0f), sil))));\n}\n";
 }
 
 // Matrix instructions of one stage, issued by one thread: level l = i + j of digit i of v and
@@ -1007,28 +1104,26 @@ std::string emit_transport_tc(const Mechanism& m, const EmitOptions& opt, const 
     s << "        if (wg == 0) { out0_[i] = KX_NAN; out1_[i] = KX_NAN; }\n";
   s << "      }\n";
   s << "      if (cy == 0 && ok && __any_sync(0xffffffffu, in && (bad || gen))) {\n";
-  if (!thermo)
-    s << "        double isig = 0.0;\n"
-      << "        if (!bad) {\n"
-      << "          double sy = 0.0;\n"
-      << fmt("          for (int j = 0; j < %d; ++j) sy = fma(Y_[(long long)j * ld + i], kx_iw[j], sy);\n", ns)
-      << "          isig = 1.0 / sy;\n"
-      << "          if (!(isig > 0.0 && isig < KX_INF)) bad = true;\n"
-      << "        }\n";
   s << "        if (in && bad) {\n"
     << "          if (wg == 0) atomicMin(&kx_bad_first, (unsigned long long)i);\n";
-  if (!diff) s << "          if (wg == 0) { out0_[i] = KX_NAN; out1_[i] = KX_NAN; }\n        } else if (in && gen && wg == 0) {\n"
-               << (visc ? fmt("          const double2 v = kx_visc_state(Y_, ld, i, kx_d2df(log(T) - %s), isig);\n", D(kTcLmid).c_str())
-                        : std::string("          const double2 v = kx_thermo_state(Y_, ld, i, T);\n"))
-               << "          out0_[i] = v.x; out1_[i] = v.y;\n        }\n";
-  else s << fmt("          for (int k = wg; k < %d; k += %d) out2_[(long long)k * ld + i] = KX_NAN;\n        }\n", ns, G)
-         << "        const kx_df Lt = kx_d2df(log(gen && !bad ? T : 1000.0) - " << D(kTcLmid) << ");\n"
-         << "        for (unsigned w = __ballot_sync(0xffffffffu, in && gen && !bad); w; w &= w - 1) {\n"
-         << "          const int src = __ffs(w) - 1;\n"
-         << fmt("          for (int k = wg; k < %d; k += %d) {\n", ns, G)
-         << "            const double d = kx_diff_row(Y_, ld, __shfl_sync(0xffffffffu, i, src), k, __shfl_sync(0xffffffffu, Lt.hi, src),\n"
-         << "                                         __shfl_sync(0xffffffffu, Lt.lo, src), __shfl_sync(0xffffffffu, P, src));\n"
-         << "            if (lane == src) out2_[(long long)k * ld + i] = d;\n          }\n        }\n";
+  if (thermo) {
+    s << "          if (wg == 0) { out0_[i] = KX_NAN; out1_[i] = KX_NAN; }\n        } else if (in && gen && wg == 0) {\n"
+      << "          const double2 v = kx_thermo_state(Y_, ld, i, T);\n          out0_[i] = v.x; out1_[i] = v.y;\n        }\n";
+  } else {
+    if (visc) s << "          if (wg == 0) { out0_[i] = KX_NAN; out1_[i] = KX_NAN; }\n        }\n";
+    else s << fmt("          for (int k = wg; k < %d; k += %d) out2_[(long long)k * ld + i] = KX_NAN;\n        }\n", ns, G);
+    // the states pair by pair, one after the other by a warp, dealt to the groups
+    s << "        const kx_df Lt = kx_d2df(log(gen && !bad ? T : 1000.0) - " << D(kTcLmid) << ");\n"
+      << "        int nth = 0;\n"
+      << "        for (unsigned w = __ballot_sync(0xffffffffu, in && gen && !bad); w; w &= w - 1, ++nth) {\n"
+      << fmt("          if ((nth & %d) != wg) continue;\n", G - 1)
+      << "          const int src = __ffs(w) - 1;\n"
+      << "          const long long is = __shfl_sync(0xffffffffu, i, src);\n"
+      << "          const float Lh = __shfl_sync(0xffffffffu, Lt.hi, src), Ll = __shfl_sync(0xffffffffu, Lt.lo, src);\n";
+    if (visc) s << "          const double2 v = kx_visc_state(Y_, ld, is, Lh, Ll);\n"
+                << "          if (lane == src) { out0_[i] = v.x; out1_[i] = v.y; }\n        }\n";
+    else s << "          kx_diff_state(Y_, ld, is, Lh, Ll, __shfl_sync(0xffffffffu, P, src), out2_);\n        }\n";
+  }
   s << "      }\n      i = in1; T = T1; P = P1;\n    }\n    asm volatile(\"cp.async.wait_all;\" ::: \"memory\");\n  }\n";
   s << "  kx_fence_before();\n  __syncthreads();\n"
     << fmt("  if (warp == %d) asm volatile(\"tcgen05.dealloc.cta_group::1.sync.aligned.b32 %%0, %d;\" ::\"r\"(tmem));\n", 4 * G, 512);

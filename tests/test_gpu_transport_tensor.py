@@ -149,3 +149,25 @@ def test_like_mass_fractions(name, kernel):
         a = a.cpu().numpy()
         err = np.abs(a - b) / (np.abs(b) if kernel != "thermo" else np.abs(b).max())
         assert err.max() <= 1e-13, f"{err.max():.2e}"
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("name", NAMES)
+def test_all_outside_the_basis(name, precision):
+    """Whole tiles below 200 K or above 4000 K: a warp per state, its lanes over the rows; nearly pure and pure ones."""
+    T, p, Y = states(name, 275)
+    T[:] = np.where(np.arange(275) % 2, 4000.0 + 10.0 * np.arange(275), 199.0 - 0.3 * np.arange(275))
+    for q, eps in enumerate((0.45, 1e-3, 1e-9)):
+        for k in range(4):   # species 2 k fills 1 - eps of the state
+            i = 20 + 4 * q + k
+            Y[:, i] *= eps / (Y[:, i].sum() - Y[2 * k, i])
+            Y[2 * k, i] = 1.0 - eps
+    Y[-3:, 80:90] = 0.0
+    check(name, T, p, Y, precision, ld_pad=5)
+    Y[:, 3] = 0.0
+    Y[4, 3] = 1.0
+    torch = torch_cuda()
+    out = [t.cpu().numpy() for t in mechanism(name).transport(*to_device(torch, T, p, Y), precision=precision)]
+    ref = oracle(name).transport(T[3:4], p[3:4], np.ascontiguousarray(Y[:, 3:4]))
+    for a, b in zip(out, ref):
+        np.testing.assert_allclose(a[..., 3:4], b, rtol=1e-12 if precision == "fp64" else 5e-6)
