@@ -81,7 +81,21 @@ def kernel_roofline(mech, name, n, ms, sm_max):
     the emitter's per-point float64 instructions against the float64 pipe, or
     its float32-pipe instructions (double-float kernels: each float-pair
     primitive at its instruction count) against the float32 pipe, whichever
-    takes longer at peak."""
+    takes longer at peak.  A swept rate kernel (most of its reactions in
+    float32) against the issue slots: the instructions that it executes, from
+    the committed capture of this exact kernel (no fraction without one), with
+    the method's work at the price of float pairs beside it as a rate."""
+    if swept(mech, name):
+        ex, work = executed_instr(mech, name), mech.op_counts(name)["fp32"]
+        peak = SMS * 128 * sm_max / 1e3
+        ach = ex * n / (ms * 1e-3) / 1e9 if ex else None
+        return {"bound": "issue", "kernel": name, "achieved": ach, "peak": peak, "unit": "G instr/s (per thread)",
+                "frac": ach / peak if ex else None, "per_point_instr": ex,
+                "peak_source": f"{SMS} SMs x 128 lanes x {sm_max:.0f} MHz (four warp instructions issued per clock, max SM clock); "
+                               "instructions executed: committed ncu capture",
+                "method_work": {"per_point": work, "rate": work * n / (ms * 1e-3) / 1e9, "unit": "G float-pair-priced instr/s",
+                                "note": "every reaction priced as float-pair work, 98 % of which the sweep does in float32: "
+                                        "work per time, not a share of a peak"}}
     f64 = ops_per_point(mech, name)
     f32 = mech.op_counts(name)["fp32"]
     p64, p32 = fp64_peak_gops(sm_max), fp32_peak_gops(sm_max)
@@ -405,7 +419,8 @@ def run_kx(args):
 
         def step_bound(knames, ms_each):
             """t_bound of the step: per kernel the slowest of its float64 instructions at the
-            float64 peak, its float32-pipe instructions at the float32 peak and its algorithmic
+            float64 peak, its float32-pipe instructions at the float32 peak (swept rate kernels:
+            the instructions executed at the issue rate) and its algorithmic
             bytes at the measured HBM copy rate; summed over the kernels of the step."""
             tb, parts = 0.0, {}
             byt = {"wdot": 8 * (2 + 2 * ns), "thermo": 8 * (2 + ns + 2), "visc": 8 * (2 + ns + 2),
@@ -414,11 +429,13 @@ def run_kx(args):
                 c = mech.op_counts(kname)
                 t64 = ops_per_point(mech, kname) * n / (fp64_peak_gops(sm_max) * 1e9)
                 t32 = c["fp32"] * n / (fp32_peak_gops(sm_max) * 1e9)
+                if swept(mech, kname):   # what it executes, at the issue rate
+                    t32 = (executed_instr(mech, kname) or 0.0) * n / (SMS * 128 * sm_max * 1e6)
                 tm = byt[kname.split("_")[0]] * n / (hbm * 1e9)
                 t = max(t64, t32, tm)
                 tb += t
                 parts[kname] = {"t_bound_ms": t * 1e3, "measured_ms": ms_k,
-                                "bound": "fp64" if t == t64 else "fp32" if t == t32 else "hbm"}
+                                "bound": "fp64" if t == t64 else "issue" if t == t32 and swept(mech, kname) else "fp32" if t == t32 else "hbm"}
             return tb * 1e3, parts
 
         roof["traffic"] = profiled_traffic(mech, names[dom], n)
@@ -451,7 +468,8 @@ def run_kx(args):
             "roofline": roof,
             "step_roofline": (lambda tb: {"t_bound_ms": tb[0], "measured_ms": ms, "frac": tb[0] / ms, "kernels": tb[1],
                                           "definition": "per kernel max(float64 instr / float64 peak, float32-pipe "
-                                                        "instr / float32 peak, algorithmic bytes / measured HBM), "
+                                                        "instr / float32 peak (swept rates: executed instr / issue "
+                                                        "peak), algorithmic bytes / measured HBM), "
                                                         "summed over the step"})(step_bound(names, per)),
             "e2e": {"value": world * n / (e2e_ms * 1e-3) / 1e6, "unit": "Mpoints/s", "api": "kx_evaluate_host",
                     "chunk": chunk,
@@ -625,6 +643,23 @@ def profiled_traffic(mech, name, n):
             d = json.load(f)
         if d.get("mechanism") == MECH and d.get("source_hash") == mech.source_hash(name):
             return d["bytes_per_state"] * n
+    return None
+
+
+def swept(mech, name):
+    """Whether a kernel is a rate kernel with the float32 sweep."""
+    return name.startswith("wdot") and "kx_msk" in mech.kernel_source(name)
+
+
+def executed_instr(mech, name):
+    """Instructions that a kernel executes per state, from the committed ncu capture of this exact kernel (matched by
+    the hash of its emitted source); None when there is none."""
+    import glob
+    for path in glob.glob(os.path.join(ROOT, "profiles", f"traffic_{name}_*.json")):
+        with open(path) as f:
+            d = json.load(f)
+        if d.get("source_hash") == mech.source_hash(name):
+            return d.get("instr_per_state")
     return None
 
 
