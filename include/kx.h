@@ -130,7 +130,7 @@ typedef struct {
                          thread-per-state kernel's resident capacity (one wave of its blocks on
                          every SM; ~155k and ~97k states on GB300) and u the share of lane slots
                          the warp-cooperative class rounds fill (~0.2 for 9/21, ~0.9 for 53/325);
-                         the crossovers measured on GB300;
+                         the crossovers measured on GB300 on those two mechanisms;
                          1 always one thread per state (species vectors in local memory);
                          2 always warp-cooperative (the states of a warp share its lanes: the
                          reactions of each class dealt out as (state, reaction) pairs, species
@@ -139,16 +139,17 @@ typedef struct {
                          not bit for bit (different summation orders). */
   int rates_group;    /* warp-cooperative production rates: states per warp, a power of two up to
                          32; 0 (default) one */
-  int vjp_form;       /* double-float adjoint, the terms d R/d C_k = nu R/C_k: 0 (default) the
-                         reaction's rate mantissa times a per-state reciprocal 1/|C_k| (log space
-                         only where the rate underflows); 1 one log-space exponential
+  int vjp_form;       /* double-float adjoint, the terms d R/d C_k = nu R/C_k: 0 (default) from
+                         the reaction's rate mantissa and power of two, times 1/|C_k| for each
+                         term or (thread per state, above 16 species) once for a species' sum;
+                         1 one log-space exponential
                          exp(ln |R| - ln |C_k|) per entry (no reciprocal table) */
   int vjp_layout;     /* double-float adjoint: 0 (default) by batch size -- the warp-cooperative
-                         kernel for batches below min(C, 8192 w u^2) states (7000 above 16 species), C the thread-per-state
-                         kernel's resident capacity, w the warp-cooperative kernel's resident warps
+                         kernel for batches below min(C, 8192 w u^2) states (7000 above 16 species),
+                         C the thread-per-state kernel's resident capacity, w the warp-cooperative kernel's resident warps
                          per SM and u the share of lane slots its class rounds fill (the crossover
-                         measured on GB300: ~8k states for 9/21, ~95k for 53/325, ~25k for
-                         160/900), one thread per state from there on; 1 always one thread per
+                         measured on GB300: ~8k states for 9/21, ~77k for 53/325, ~25k for
+                         160/900; the rule gives 6k, 95k and 25k), one thread per state from there on; 1 always one thread per
                          state; 2 always warp-cooperative (one state per warp, its vectors and
                          per-reaction terms in shared memory, d/dC_k gathered species-major;
                          mechanisms whose warp slice exceeds 50 KB keep one thread per state
@@ -156,8 +157,8 @@ typedef struct {
                          entry's term scale, not bit for bit. */
   int rates_negligible; /* double-float KX_FP64 production rates: 0 (default) a reaction whose rate
                          is below 2^-40 of its state's largest (above 64 species or 400
-                         reactions: for every state of a warp) is evaluated in float32 (its error is far inside the per-point bar, but a
-                         species all of whose reactions are that small gets wdot_k to ~1e-4 of
+                         reactions: for every state of a warp) is evaluated in float32 (its
+                         error is far inside the per-point bar, but a species all of whose reactions are that small gets wdot_k to ~1e-4 of
                          itself); 1 every reaction in float pairs (wdot_k to ~1e-11 of the
                          species' own gross rate, for the species within 1e-40 of their state's
                          largest rate: for finite differences of the rates) */

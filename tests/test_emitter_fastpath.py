@@ -1,5 +1,7 @@
 """Host-side checks of the emitted float32 path of the float-pair rate
-kernels (no GPU): the path is a warp-wide vote on float32 estimates against
+kernels' class loops and warp rounds (no GPU; up to 64 species and 400
+reactions the thread-per-state kernel runs those loops only for warps with
+large negative mass fractions, behind the sweep): the path is a warp-wide vote on float32 estimates against
 2^-40 of the state's scale anchor, emitted for the elementary, three-body,
 falloff and chemically activated classes of the production-rate kernels
 only (never in the rates-of-progress kernel, whose bar is each reaction's

@@ -1,5 +1,8 @@
-"""The share of reaction-warps that the float-pair rate kernel's float32 path
-takes on the benchmark's states, reproduced on the host: the oracle's gross
+"""The share of reaction-warps that the class loops' float32 path (a vote of
+each warp; mechanisms above 64 species or 400 reactions, the no-alloc kernel,
+and warps with large negative mass fractions of smaller ones, whose default
+is the sweep with each state's own choice) would take on the benchmark's
+states if it ran them, reproduced on the host: the oracle's gross
 rates of each reaction, visited in the emitted kernel's class order, with
 the kernel's running per-state scale (set by the first rate at 2^62, raised
 when a rate lands above 2^96) and its rule (every state of a warp of 32

@@ -1,6 +1,7 @@
-"""The float-pair rate kernel's float32 path: a reaction whose rate is below
-2^-40 of its state's scale anchor, for every state of a warp, is evaluated in
-float32.  A state's results therefore depend, within the float64 bar, on the
+"""The float-pair rate kernels' float32 path: a reaction whose rate is below
+2^-40 of its state's largest is evaluated in float32, by each state's own
+choice (the sweep) or where it holds for every state of a warp (the class
+loops), so that a state's results may depend, within the float64 bar, on the
 states that share its warp: the same states under other warp groupings
 (the batch shifted by 1, 13 and 31 states) must agree to 1e-10 of the
 per-point scale, and each grouping must meet that bar against the oracle on
