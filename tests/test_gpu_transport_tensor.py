@@ -153,10 +153,14 @@ def test_like_mass_fractions(name, kernel):
 
 @pytest.mark.parametrize("precision", ["fp64", "mixed"])
 @pytest.mark.parametrize("name", NAMES)
-def test_all_outside_the_basis(name, precision):
-    """Whole tiles below 200 K or above 4000 K: a warp per state, its lanes over the rows; nearly pure and pure ones."""
+@pytest.mark.parametrize("share", [1.0, 0.45, 0.1])
+def test_outside_the_basis(name, precision, share):
+    """Tiles of states below 200 K or above 4000 K, all of them or among others: a warp per state, its lanes over the
+    rows; nearly pure and pure states."""
     T, p, Y = states(name, 275)
-    T[:] = np.where(np.arange(275) % 2, 4000.0 + 10.0 * np.arange(275), 199.0 - 0.3 * np.arange(275))
+    out = np.where(np.arange(275) % 2, 4000.0 + 10.0 * np.arange(275), 199.0 - 0.3 * np.arange(275))
+    T = np.where(np.random.default_rng(7).random(275) < share, out, T)
+    T[3] = 4500.0
     for q, eps in enumerate((0.45, 1e-3, 1e-9)):
         for k in range(4):   # species 2 k fills 1 - eps of the state
             i = 20 + 4 * q + k
